@@ -313,11 +313,13 @@ __global__ void k_inverse_row(const FrontDesc<C>* fd, int i) {
     for (int u = 0; u < 4; ++u) ot[r + (cg * 4 + u) * TILE] = cneg(out[u]);
 }
 
-// Copy L21 (rows nown..m-1, columns 0..nown-1 of the front) into packed tiles.
+// Copy the front's rows nown..m-1, columns 0..nown-1 into packed tiles, for the fronts whose tc
+// flag is `which`: L21 of a front factored by the panel steps alone (0), or the M21 that the
+// tensor-core product left there (1).
 template <class C>
-__global__ void k_pack_l21(const FrontDesc<C>* fd) {
+__global__ void k_pack_l21(const FrontDesc<C>* fd, int which) {
     const FrontDesc<C>& f = fd[blockIdx.y];
-    if (f.tc) return;   // written by the tensor-core L21 product
+    if (f.tc != which) return;
     const int own_t = cdiv_dev(f.nown, TILE), upd_t = cdiv_dev(f.nupd, TILE);
     const int q = blockIdx.x;
     if (q >= own_t * upd_t) return;
@@ -332,12 +334,53 @@ __global__ void k_pack_l21(const FrontDesc<C>* fd) {
     }
 }
 
+// M21 = L21 L11^{-1} of a front factored by the panel steps alone, straight into the packed tiles:
+// tile (rt, j) = sum over k >= j of L21(rt, k) (from the front) times L11^{-1}(k, j) (packed).
+template <class C>
+__global__ void k_m21(const FrontDesc<C>* fd) {
+    const FrontDesc<C>& f = fd[blockIdx.y];
+    if (f.tc) return;
+    const int own_t = cdiv_dev(f.nown, TILE), upd_t = cdiv_dev(f.nupd, TILE);
+    const int q = blockIdx.x;
+    if (q >= own_t * upd_t) return;
+    const int rt = q / own_t, j = q % own_t;
+    __shared__ C A[TILE][TILE + 1];   // A[k][r]: L21(rt, kt)
+    __shared__ C B[TILE][TILE + 1];   // B[k][c]: L11^{-1}(kt, j)
+    const int t = threadIdx.x;
+    const int r = t % TILE, cg = t / TILE;
+    C acc[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc[u] = czero<C>();
+    for (int kt = j; kt < own_t; ++kt) {
+        const C* xt = f.fac + (f.linv_off + tri_index(kt, j)) * TILE2;
+        for (int e = t; e < TILE2; e += blockDim.x) {
+            const int rr = e % TILE, kk = e / TILE;
+            const int row = rt * TILE + rr, col = kt * TILE + kk;
+            C v = czero<C>();
+            if (row < f.nupd && col < f.nown) v = f.F[(long long)(f.nown + row) + (long long)col * f.m];
+            A[kk][rr] = v;
+            B[e % TILE][e / TILE] = xt[e];
+        }
+        __syncthreads();
+        for (int kk = 0; kk < TILE; ++kk) {
+            const C av = A[kk][r];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) cfma(acc[u], av, B[kk][cg * 4 + u]);
+        }
+        __syncthreads();
+    }
+    C* ot = f.fac + (f.l21_off + (long long)q) * TILE2;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) ot[r + (cg * 4 + u) * TILE] = acc[u];
+}
+
 }  // namespace
 
 // Kernel kinds of the factorization, for the optional per-kind timing (HZ_FACTOR_PROFILE=1).
-enum { FK_ASSEMBLE, FK_EXTEND, FK_DIAG, FK_PANEL, FK_UPDATE, FK_INVERSE, FK_GEMM_L21, FK_GEMM_SCHUR, FK_PACK, FK_N };
+enum { FK_ASSEMBLE, FK_EXTEND, FK_DIAG, FK_PANEL, FK_UPDATE, FK_INVERSE, FK_GEMM_L21, FK_GEMM_SCHUR, FK_GEMM_M21, FK_M21, FK_PACK, FK_N };
 const char* const kFactorKindNames[FK_N] = {"k_assemble", "k_extend_add", "k_diag", "k_panel", "k_update",
-                                            "k_inverse_row", "k_front_gemm L21", "k_front_gemm Schur", "k_pack_l21"};
+                                            "k_inverse_row", "k_front_gemm L21", "k_front_gemm Schur",
+                                            "k_front_gemm M21", "k_m21", "k_pack_l21"};
 
 template <class C>
 void factor_layers(Ctx& ctx) {
@@ -404,6 +447,7 @@ void factor_layers(Ctx& ctx) {
                 std::vector<FrontGemmDesc> gds;
                 std::vector<ExtDesc<C>> eds[2];
                 int max_nasm = 0, max_own = 0, max_rt = 0, max_tri = 0, max_pack = 0, max_ext = 0;
+                int max_pack_tc = 0;
                 for (int l = g0; l < g1; ++l) {
                     Layer& ly = ctx.layers[l];
                     Shape& sh = ctx.shapes[ly.shape];
@@ -440,7 +484,8 @@ void factor_layers(Ctx& ctx) {
                         max_rt = std::max(max_rt, cdiv(std::max(rows, 0), TILE));
                         int T = cdiv(std::max(rows, 0), TILE);
                         max_tri = std::max(max_tri, T * (T + 1) / 2);
-                        if (!f.tc) max_pack = std::max(max_pack, nd.own_t * nd.upd_t);
+                        int& mp = f.tc ? max_pack_tc : max_pack;
+                        mp = std::max(mp, nd.own_t * nd.upd_t);
                         for (int k = 0; k < nd.nchild; ++k) {
                             const Node& ch = sh.nodes[nd.child[k]];
                             ExtDesc<C> e;
@@ -524,13 +569,13 @@ void factor_layers(Ctx& ctx) {
                     HZ_CHECK_LAUNCH();
                     FP_END(FK_INVERSE);
                 }
-                // 5. tensor-core fronts: L21 = F21 L11^{-T} D^{-1} into the packed tiles, then the
-                //    Schur complement F22 -= L21 D L21^T
+                // 5. tensor-core fronts: L21 = F21 L11^{-T} D^{-1} into the packed tiles, the Schur
+                //    complement F22 -= L21 D L21^T, then M21 = L21 L11^{-1}, packed over L21
                 if (!gds.empty()) {
-                    std::vector<GemmItem> it_l21, it_schur;
-                    front_gemm_items(gds, it_l21, it_schur);
+                    std::vector<GemmItem> it_l21, it_schur, it_m21;
+                    front_gemm_items(gds, it_l21, it_schur, it_m21);
                     const size_t need_g = gds.size() * sizeof(FrontGemmDesc);
-                    const size_t need_i = (it_l21.size() + it_schur.size()) * sizeof(GemmItem);
+                    const size_t need_i = (it_l21.size() + it_schur.size() + it_m21.size()) * sizeof(GemmItem);
                     if (need_g > gd_cap) {
                         if (d_gd) cudaFree(d_gd);
                         gd_cap = need_g * 2;
@@ -547,6 +592,8 @@ void factor_layers(Ctx& ctx) {
                                             cudaMemcpyHostToDevice, st));
                     HZ_CUDA(cudaMemcpyAsync(d_items + it_l21.size(), it_schur.data(), it_schur.size() * sizeof(GemmItem),
                                             cudaMemcpyHostToDevice, st));
+                    GemmItem* d_m21 = d_items + it_l21.size() + it_schur.size();
+                    HZ_CUDA(cudaMemcpyAsync(d_m21, it_m21.data(), it_m21.size() * sizeof(GemmItem), cudaMemcpyHostToDevice, st));
                     FP_BEGIN();
                     launch_front_gemm(0, d_items, (long long)it_l21.size(), (const FrontGemmDesc*)d_gd, ctx.d_flag + 1,
                                       ctx.tc_wait_polls, st);
@@ -555,13 +602,23 @@ void factor_layers(Ctx& ctx) {
                     launch_front_gemm(1, d_items + it_l21.size(), (long long)it_schur.size(), (const FrontGemmDesc*)d_gd,
                                       ctx.d_flag + 1, ctx.tc_wait_polls, st);
                     FP_END(FK_GEMM_SCHUR);
-                }
-                // 6. pack L21 (fronts factored by the panel steps alone)
-                if (max_pack > 0) {
                     FP_BEGIN();
-                    k_pack_l21<C><<<dim3(max_pack, nf), 256, 0, st>>>(d_fd);
+                    launch_front_gemm(2, d_m21, (long long)it_m21.size(), (const FrontGemmDesc*)d_gd, ctx.d_flag + 1,
+                                      ctx.tc_wait_polls, st);
+                    FP_END(FK_GEMM_M21);
+                    FP_BEGIN();
+                    k_pack_l21<C><<<dim3(max_pack_tc, nf), 256, 0, st>>>(d_fd, 1);
                     HZ_CHECK_LAUNCH();
                     FP_END(FK_PACK);
+                }
+                // 6. fronts factored by the panel steps alone: pack L21, or form M21 where the
+                //    substitution (complex64) uses it
+                if (max_pack > 0) {
+                    FP_BEGIN();
+                    if (ctx.has_m21()) k_m21<C><<<dim3(max_pack, nf), 256, 0, st>>>(d_fd);
+                    else k_pack_l21<C><<<dim3(max_pack, nf), 256, 0, st>>>(d_fd, 0);
+                    HZ_CHECK_LAUNCH();
+                    FP_END(ctx.has_m21() ? FK_M21 : FK_PACK);
                 }
                 HZ_CUDA(cudaStreamSynchronize(st));
             }

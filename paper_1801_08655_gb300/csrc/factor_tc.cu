@@ -2,18 +2,23 @@
 // "Local Solves: Parallel Multi-frontal Methods" section) for complex64 fronts.
 //
 // A front F = [F11 F21^T; F21 F22] (own unknowns first, column-major, lower triangle) is
-// factored in three steps once its pivot block F11 = L11 D L11^T has been factored and L11
+// factored in these steps once its pivot block F11 = L11 D L11^T has been factored and L11
 // inverted (the CUDA-core kernels of factor.cu, FP64 pivot blocks):
 //   L21  = F21 L11^{-T} D^{-1}          (GEMM_L21: A = F21 from the front, B = L11^{-1} packed
 //                                        tiles; the output goes straight into the packed L21
 //                                        tiles of the factor storage, scaled by D^{-1} per column)
 //   F22 -= L21 D L21^T                  (GEMM_SCHUR: A = L21, B = L21 scaled by D(k) per
 //                                        reduction index; lower 128 x 128 output tiles only)
+//   M21  = L21 L11^{-1}                 (GEMM_M21: A = packed L21, B = L11^{-1} transposed; the
+//                                        output goes over F21 in the front, free by now, and is
+//                                        packed from there over L21: the substitution wants M21)
 // so the Schur update reads F22 once (K = the number of own unknowns) instead of once per
-// 32-column panel.  Both are complex products C = sum_k A(i,k) B(j,k) (no conjugation): four
+// 32-column panel.  All are complex products C = sum_k A(i,k) B(j,k) (no conjugation): four
 // real products, each with a three-term TF32 split of both operands (hi*hi + hi*lo + lo*hi)
 // and FP32 accumulation in tensor memory, i.e. FP32-level accuracy, as in the substitution
-// kernels (tc_common.cuh).
+// kernels (tc_common.cuh); the hi x lo terms have accumulators of their own (all 512 tensor-memory
+// columns are used), which halves the error of a 56^3 local solve (3.1e-5 -> 1.6e-5 of the FP64
+// one) at the same MMAs.
 //
 // One block per 128 x 128 output tile (416 threads): 4 loader warps (cp.async into a two-deep
 // raw ring: 16-byte copies of packed tiles, 8-byte copies of front columns, zero-filled beyond
@@ -35,13 +40,14 @@ namespace {
 
 using namespace tcc;
 
-enum { GEMM_L21 = 0, GEMM_SCHUR = 1 };
+enum { GEMM_L21 = 0, GEMM_SCHUR = 1, GEMM_M21 = 2 };
 
 constexpr int GN = 128;                         // output columns per item (N of the MMA)
 constexpr int G_AMAT = MR * KC * 4;             // one converted real operand matrix (8 KB)
 constexpr int G_CONV = 4 * G_AMAT + 4 * G_AMAT; // A (re/im x hi/lo) and B (re/im x hi/lo)
 constexpr int G_RAW_A = 4 * KC * 32 * 8;        // 128 rows x 16 k complex, [tile][k][row]
-constexpr int G_RAW = 2 * G_RAW_A + KC * 8;     // A, B and the 16 D(k) of the stage
+constexpr int G_RAW_B = 4 * 32 * TROW;          // B: as A, or (M21) [tile][column][k], rows padded to TROW
+constexpr int G_RAW = G_RAW_A + G_RAW_B + KC * 8;   // A, B and the 16 D(k) of the stage
 constexpr int G_BAR_OFF = 2 * G_CONV + 2 * G_RAW;
 constexpr int G_SMEM = G_BAR_OFF + 8 * 8 + 16;
 constexpr int G_THREADS = NLOAD + NCONV + 32;
@@ -63,17 +69,17 @@ __device__ __forceinline__ void load_packed(unsigned char* dst0, const float2* f
     }
 }
 
-// raw [tile][k][row] (128 rows x 16 k complex) -> split operand matrices at cv + {0,1,2,3} * G_AMAT
+// raw [tile][k][row] (128 rows x 16 k complex; TR: [tile][row][k]) -> split operand matrices at cv + {0,1,2,3} * G_AMAT
 // (re_hi, re_lo, im_hi, im_lo), optionally multiplied by d[k] first
-template <bool SCALE>
+template <bool SCALE, bool TR = false>
 __device__ __forceinline__ void convert_operand(const unsigned char* rb, const float2* d, unsigned char* cv, int ct) {
     for (int id = ct; id < MR * 4; id += NCONV) {
         const int row = id & 127, kq = id >> 7;
-        const float2* src = (const float2*)(rb + (row >> 5) * 4096);
+        const float2* src = (const float2*)(TR ? rb + row * TROW : rb + (row >> 5) * 4096);
         float re[4], im[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            float2 a = src[(4 * kq + j) * 32 + (row & 31)];
+            float2 a = TR ? src[4 * kq + j] : src[(4 * kq + j) * 32 + (row & 31)];
             if (SCALE) {
                 const float2 s = d[4 * kq + j];
                 a = make_float2(a.x * s.x - a.y * s.y, a.x * s.y + a.y * s.x);
@@ -114,7 +120,7 @@ k_front_gemm(const GemmItem* __restrict__ items, const FrontGemmDesc* __restrict
     const int mma_warp = (NLOAD + NCONV) / 32;
 
     if (w == mma_warp) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(tptr)), "r"(2 * GN));
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(tptr)), "r"(4 * GN));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (t == 0) {
@@ -141,7 +147,7 @@ k_front_gemm(const GemmItem* __restrict__ items, const FrontGemmDesc* __restrict
             if (s >= 2) ok = mbar_wait(smem_u32(raw_empty + slot), (uint32_t)((use - 1) & 1), abort, polls);
             if (!ok) break;
             unsigned char* rb = raw + slot * G_RAW;
-            const int kt = s >> 1, hk = s & 1;
+            const int kt = (s >> 1) + (MODE == GEMM_M21 ? it.tj * 4 : 0), hk = s & 1;
             if (MODE == GEMM_L21) {
                 // A: F21 rows i0 .. i0+127, columns kt*32 + hk*16 .. +15 (8-byte copies)
 #pragma unroll 4
@@ -162,13 +168,25 @@ k_front_gemm(const GemmItem* __restrict__ items, const FrontGemmDesc* __restrict
                 load_packed(rb, f.fac, it.ti * 4, hk, t, [&](int rt) -> long long {
                     return rt < f.upd_t ? f.l21_off + (long long)rt * f.own_t + kt : -1;
                 });
+                if (MODE == GEMM_M21) {
+                    // B(j, k) = L11^{-1}(k, j): column j of tile (kt, j / 32), 16 consecutive k (128 bytes)
+                    for (int c = t; c < 1024; c += NLOAD) {
+                        const int oi = c >> 8, r = (c >> 3) & 31, jj = c & 7;
+                        const int ct = it.tj * 4 + oi;
+                        const bool in = ct < f.own_t && ct <= kt;
+                        const float2* src = f.fac + (f.linv_off + (in ? tri_idx(kt, ct) : 0)) * TILE2 + 32 * r + hk * KC + jj * 2;
+                        cp16(smem_u32(rb + G_RAW_A + (oi * 32 + r) * TROW + jj * 16), src, in ? 16 : 0);
+                    }
+                    cp_async_arrive(raw_full + slot);
+                    continue;
+                }
                 load_packed(rb + G_RAW_A, f.fac, it.tj * 4, hk, t, [&](int rt) -> long long {
                     return rt < f.upd_t ? f.l21_off + (long long)rt * f.own_t + kt : -1;
                 });
                 if (t < KC) {   // D(k) from the front's diagonal
                     const int col = kt * TILE + hk * KC + t;
                     const bool in = col < f.nown;
-                    cp8(smem_u32(rb + 2 * G_RAW_A + t * 8), in ? (const void*)(f.F + (long long)col * (f.m + 1)) : (const void*)f.F,
+                    cp8(smem_u32(rb + G_RAW_A + G_RAW_B + t * 8), in ? (const void*)(f.F + (long long)col * (f.m + 1)) : (const void*)f.F,
                         in ? 8 : 0);
                 }
             }
@@ -186,7 +204,8 @@ k_front_gemm(const GemmItem* __restrict__ items, const FrontGemmDesc* __restrict
             const unsigned char* rb = raw + slot * G_RAW;
             unsigned char* cv = conv + slot * G_CONV;
             convert_operand<false>(rb, nullptr, cv, ct);
-            if (MODE == GEMM_SCHUR) convert_operand<true>(rb + G_RAW_A, (const float2*)(rb + 2 * G_RAW_A), cv + 4 * G_AMAT, ct);
+            if (MODE == GEMM_SCHUR) convert_operand<true>(rb + G_RAW_A, (const float2*)(rb + G_RAW_A + G_RAW_B), cv + 4 * G_AMAT, ct);
+            else if (MODE == GEMM_M21) convert_operand<false, true>(rb + G_RAW_A, nullptr, cv + 4 * G_AMAT, ct);
             else convert_operand<false>(rb + G_RAW_A, nullptr, cv + 4 * G_AMAT, ct);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_arrive(raw_empty + slot);
@@ -199,7 +218,7 @@ k_front_gemm(const GemmItem* __restrict__ items, const FrontGemmDesc* __restrict
             ok = mbar_wait(smem_u32(conv_full + cb), (uint32_t)(use & 1), abort, polls);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            mma_stage<GN, 3>(smem_u32(conv + cb * G_CONV), tm_r, tm_i, s == 0);
+            mma_stage<GN, 3, true>(smem_u32(conv + cb * G_CONV), tm_r, tm_i, s == 0);
             mma_commit(conv_empty + cb);
             *committed = s + 1;
         }
@@ -230,6 +249,15 @@ k_front_gemm(const GemmItem* __restrict__ items, const FrontGemmDesc* __restrict
         for (int c0 = sub * (GN / 2); c0 < (sub + 1) * (GN / 2); c0 += 16) {
             uint32_t vr[16], vi[16];
             tmem_ld16(tm_r + lane_off + (uint32_t)c0, tm_i + lane_off + (uint32_t)c0, vr, vi);
+            {   // the hi x lo terms' accumulators
+                uint32_t lr_[16], li_[16];
+                tmem_ld16(tm_r + 2 * GN + lane_off + (uint32_t)c0, tm_i + 2 * GN + lane_off + (uint32_t)c0, lr_, li_);
+#pragma unroll
+                for (int jj = 0; jj < 16; ++jj) {
+                    vr[jj] = __float_as_uint(__uint_as_float(vr[jj]) + __uint_as_float(lr_[jj]));
+                    vi[jj] = __float_as_uint(__uint_as_float(vi[jj]) + __uint_as_float(li_[jj]));
+                }
+            }
             if (MODE == GEMM_L21) {
                 const int rt = i >> 5;
                 if (rt < f.upd_t) {
@@ -242,6 +270,15 @@ k_front_gemm(const GemmItem* __restrict__ items, const FrontGemmDesc* __restrict
                         const float a = __uint_as_float(vr[jj]), b = __uint_as_float(vi[jj]);
                         f.fac[(f.l21_off + (long long)rt * f.own_t + ctile) * TILE2 + (i & 31) + (j & 31) * TILE] =
                             make_float2(a * d.x - b * d.y, a * d.y + b * d.x);
+                    }
+                }
+            } else if (MODE == GEMM_M21) {
+                if (i < f.nupd) {
+#pragma unroll
+                    for (int jj = 0; jj < 16; ++jj) {
+                        const int j = it.tj * GN + c0 + jj;
+                        if (j < f.nown)
+                            f.F[(long long)(f.nown + i) + (long long)j * f.m] = make_float2(__uint_as_float(vr[jj]), __uint_as_float(vi[jj]));
                     }
                 }
             } else if (i < f.nupd) {
@@ -261,17 +298,19 @@ k_front_gemm(const GemmItem* __restrict__ items, const FrontGemmDesc* __restrict
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (w == mma_warp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(2 * GN));
+    if (w == mma_warp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(4 * GN));
 }
 
 }  // namespace
 
 bool front_gemm_eligible(int nown, int nupd, int min_upd) { return nupd >= min_upd && nown >= TILE; }
 
-// Work items of the two products for the given fronts (longest reductions first).
-void front_gemm_items(const std::vector<FrontGemmDesc>& fr, std::vector<GemmItem>& l21, std::vector<GemmItem>& schur) {
+// Work items of the three products for the given fronts (longest reductions first).
+void front_gemm_items(const std::vector<FrontGemmDesc>& fr, std::vector<GemmItem>& l21, std::vector<GemmItem>& schur,
+                      std::vector<GemmItem>& m21) {
     l21.clear();
     schur.clear();
+    m21.clear();
     for (int q = 0; q < (int)fr.size(); ++q) {
         const FrontGemmDesc& f = fr[q];
         const int T = cdiv(f.nupd, MR), J = cdiv(f.nown, GN);
@@ -279,6 +318,7 @@ void front_gemm_items(const std::vector<FrontGemmDesc>& fr, std::vector<GemmItem
             for (int tj = 0; tj < J; ++tj) {
                 const int kend = std::min((tj + 1) * (GN / TILE), f.own_t);
                 l21.push_back({q, ti, tj, 2 * kend});
+                m21.push_back({q, ti, tj, 2 * (f.own_t - tj * (GN / TILE))});
             }
             for (int tj = 0; tj <= ti; ++tj) schur.push_back({q, ti, tj, 2 * f.own_t});
         }
@@ -286,25 +326,21 @@ void front_gemm_items(const std::vector<FrontGemmDesc>& fr, std::vector<GemmItem
     auto longer = [](const GemmItem& a, const GemmItem& b) { return a.nst > b.nst; };
     std::stable_sort(l21.begin(), l21.end(), longer);
     std::stable_sort(schur.begin(), schur.end(), longer);
+    std::stable_sort(m21.begin(), m21.end(), longer);
 }
 
 void launch_front_gemm(int mode, const GemmItem* d_items, long long n, const FrontGemmDesc* d_fronts, int* flag,
                        long long polls, cudaStream_t st) {
     if (n <= 0) return;
-    static bool attr[2] = {false, false};
+    static bool attr[3] = {false, false, false};
+    auto* kern = mode == GEMM_L21 ? k_front_gemm<GEMM_L21> : mode == GEMM_SCHUR ? k_front_gemm<GEMM_SCHUR> : k_front_gemm<GEMM_M21>;
     if (!attr[mode]) {
-        if (mode == GEMM_L21)
-            HZ_CUDA(cudaFuncSetAttribute(k_front_gemm<GEMM_L21>, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM));
-        else
-            HZ_CUDA(cudaFuncSetAttribute(k_front_gemm<GEMM_SCHUR>, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM));
+        HZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM));
         attr[mode] = true;
     }
     for (long long b0 = 0; b0 < n; b0 += 65535LL * 16) {
         const unsigned grid = (unsigned)std::min<long long>(n - b0, 65535LL * 16);
-        if (mode == GEMM_L21)
-            k_front_gemm<GEMM_L21><<<grid, G_THREADS, G_SMEM, st>>>(d_items + b0, d_fronts, flag, polls);
-        else
-            k_front_gemm<GEMM_SCHUR><<<grid, G_THREADS, G_SMEM, st>>>(d_items + b0, d_fronts, flag, polls);
+        kern<<<grid, G_THREADS, G_SMEM, st>>>(d_items + b0, d_fronts, flag, polls);
         HZ_CHECK_LAUNCH();
     }
 }

@@ -29,6 +29,11 @@ struct LayerCoef {
     double omega2, inv_h2;
 };
 
+// One vector to clear (launch_zero): 8-byte aligned pointer, a multiple of 8 bytes.
+struct ZeroDev { void* p; long long bytes; };
+// Clears n vectors, the longest of max_bytes, in one launch.
+void launch_zero(const ZeroDev* d, int n, long long max_bytes, cudaStream_t st);
+
 // A set of layers solved together (one job per layer) with its per-level task lists.
 struct Batch {
     std::vector<int> layers;
@@ -48,7 +53,9 @@ struct Batch {
     std::vector<long long> pair_off[4], pair_cnt[4];  // tensor-core tasks: two output tiles each
     Task* d_tasks = nullptr;
     void* d_jobs = nullptr;                     // JobDev<C>[njobs]
-    std::vector<std::pair<void*, void*>> vec_ptrs;  // (acc, x) of each job
+    std::vector<std::pair<void*, void*>> vec_ptrs;  // (acc, x) of each layer
+    ZeroDev* d_zero[2] = {nullptr, nullptr};        // acc / x vectors of every layer, for launch_zero
+    long long zero_max = 0;                         // bytes of the longest of them
     std::vector<long long> vec_rows;
     double alg_bytes = 0;       // factor bytes one forward+backward substitution streams (all jobs)
     double flops_per_col = 0;   // real flops per right-hand-side column (all jobs)
@@ -235,12 +242,17 @@ struct Ctx {
     std::map<std::tuple<int, int, int>, KernStat> kern_lvl;  // per (kind, phase, tree level)
     std::string prof_text;
     TraceBlocks tb;
+    // complex64 substitutions run on M21 = L21 L11^{-1} (solve.cu) and leave the solution in the
+    // layer's accumulator slot; complex128 ones on L21, with the solution in the x slot
+    bool has_m21() const { return prec != HZ_PREC_FP64; }
+    void* result(int l) const { return has_m21() ? slot_acc[l] : slot_x[l]; }
 };
 
 template <class C> void factor_layers(Ctx& ctx);
 
 // Tensor-core products of the factorization of complex64 fronts (factor_tc.cu): L21 = F21 L11^{-T}
-// D^{-1} into the packed factor tiles, then F22 -= L21 D L21^T in the front.
+// D^{-1} into the packed factor tiles, F22 -= L21 D L21^T in the front, and M21 = L21 L11^{-1} over the
+// front's F21 (launch_front_gemm modes 0, 1, 2).
 struct FrontGemmDesc {
     float2* F;             // dense front (m x m, column-major)
     float2* fac;           // layer's packed factor tiles
@@ -251,7 +263,7 @@ struct FrontGemmDesc {
 struct GemmItem { int front, ti, tj, nst; };   // 128 x 128 output tile (ti, tj), pipeline stages
 bool front_gemm_eligible(int nown, int nupd, int min_upd);
 void front_gemm_items(const std::vector<FrontGemmDesc>& fronts, std::vector<GemmItem>& l21,
-                      std::vector<GemmItem>& schur);
+                      std::vector<GemmItem>& schur, std::vector<GemmItem>& m21);
 void launch_front_gemm(int mode, const GemmItem* d_items, long long n, const FrontGemmDesc* d_fronts, int* flag,
                        long long polls, cudaStream_t st);
 

@@ -746,11 +746,15 @@ inline double2* pair_ptr(double2* base, const Ctx& c, int dir, int j) {
 
 template <class C>
 void rec_zero_slots(Ctx& ctx, Rec& rec, const std::vector<int>& layers, int ldc) {
+    std::vector<ZeroDev> zd;
+    long long most = 0;
     for (int l : layers) {
-        void* p = ctx.slot_acc[l];
-        const size_t bytes = (size_t)ctx.shapes[ctx.layers[l].shape].N * ldc * sizeof(C);
-        rec.add([p, bytes](cudaStream_t st) { HZ_CUDA(cudaMemsetAsync(p, 0, bytes, st)); });
+        zd.push_back({ctx.slot_acc[l], ctx.shapes[ctx.layers[l].shape].N * ldc * (long long)sizeof(C)});
+        most = std::max(most, zd.back().bytes);
     }
+    const ZeroDev* d = rec.up(zd);
+    const int n = (int)zd.size();
+    rec.add([=](cudaStream_t st) { launch_zero(d, n, most, st); });
 }
 
 // approx: the substitution serves the preconditioner, whose tensor-core products then run with
@@ -820,7 +824,7 @@ Extract<C> make_extract(Ctx& ctx, int l, bool bottom, int pl, const std::vector<
     const Layer& ly = ctx.layers[l];
     const Shape& sh = ctx.shapes[ly.shape];
     Extract<C> e;
-    e.x = (const C*)ctx.slot_x[l];
+    e.x = (const C*)ctx.result(l);
     e.pos = sh.d_pos;
     e.dst = dst;
     e.rstride = rstride;
@@ -1373,7 +1377,7 @@ void rec_reconstruct(Ctx& ctx, Rec& rec, const double2* g, bool scale, const dou
     for (int l : layers) {
         const Layer& ly = ctx.layers[l];
         VolIO<C> q;
-        q.vec = (C*)ctx.slot_x[l];
+        q.vec = (C*)ctx.result(l);
         q.pos = ctx.shapes[ly.shape].d_pos;
         q.ldc = ldc; q.col0 = 0; q.lo = ly.lo; q.hi = ly.hi; q.zlo = ly.zlo;
         io.push_back(q);
@@ -1405,7 +1409,7 @@ void op_layer_solve(Ctx& ctx, int ell, const double2* g, int ncols, double2* w) 
     rec_zero_slots<C>(ctx, rec, one, ldc);
     dim3 grid(cdiv(sh.N, 256), ncols);
     C* acc = (C*)ctx.slot_acc[ell];
-    const C* xv = (const C*)ctx.slot_x[ell];
+    const C* xv = (const C*)ctx.result(ell);
     const int* pos = sh.d_pos;
     const long long N = sh.N;
     rec.add([=](cudaStream_t st) {

@@ -2,19 +2,28 @@
 //
 // This is the local solve w = (H^l)^{-1} g that every step of the online phase calls
 // (Algorithm 2 local and inner solves; Algorithms 4-9 in the sweeps and the blocks of the
-// polarized matrix).  With the diagonal blocks of the fronts stored inverted, each tree
-// node costs four dense products on a block of columns:
+// polarized matrix).  With the diagonal blocks of the fronts stored inverted, each tree node
+// costs four dense products on a block of columns.  Complex64 factors store M21 = L21 L11^{-1}
+// in place of L21 (M21 = F21 F11^{-1}, so the node's own unknowns need no triangular solve inside
+// the recursion):
+//   forward  (leaves -> root):  acc[upd] -= M21 acc[own]            FB, level by level
+//   all nodes at once:          x[own]    = D^{-1} L^{-1} acc[own]  FA, one launch
+//                               acc[own]  = L^{-T} x[own]           BB, one launch
+//   backward (root -> leaves):  acc[own] -= M21^T acc[upd]          BA, level by level
+// and the solution is left in acc.  That is 2 (H - 1) + 2 dependent phases for a tree of H levels
+// where L21 needs 4 H, with the same flops and factor bytes; the phases that leave the recursion
+// (half of them, and the ones with the shortest reductions) fill the GPU however few nodes a
+// level has.  Whole solves, L21 against M21: 24^3 with 1 column 2.60 -> 1.95 ms, 64^3 with 16
+// columns 99.3 -> 80.3 ms, with 128 columns 283 -> 204 ms.  Complex128 factors, whose products are bound by the FP64 pipe at any size, keep L21:
 //   forward  (leaves -> root):  z = Linv * acc[own];         acc[upd] -= L21 * z   (scatter)
 //   backward (root -> leaves):  v = Dinv z - L21^T x[upd];   x[own]   = Linv^T * v
-// Nodes of equal height are independent; a launch covers one phase of one height for all
-// layers of a batch.  Every block computes a TILE-row slab of one product for a chunk of
-// CC right-hand-side columns over a range of at most KS reduction tiles (split-K keeps the
-// top of the tree, where a level has few nodes with long reductions, spread over the whole
-// GPU).  Outputs are zeroed beforehand; a task covering the whole reduction of its rows stores
-// them, split reductions and FB's update rows (shared between the nodes of a level) accumulate
-// with atomics.  The factor tile stream is the HBM traffic that bounds the kernel at small
-// column counts.  Complex64 blocks of >= 64 columns can instead run on the tensor-core kernels
-// of subst_tc.cu; the autotuner decides per batch signature.
+// Every block computes a TILE-row slab of one product for a chunk of CC right-hand-side columns
+// over a range of at most KS reduction tiles (split-K keeps the top of the tree, where a level has
+// few nodes with long reductions, spread over the whole GPU).  Stored outputs are zeroed
+// beforehand; a task covering the whole reduction of its rows stores them, split reductions and
+// the updates (FB, complex64 BA) accumulate with atomics.  The factor tile stream is the HBM
+// traffic that bounds the kernel at small column counts.  Complex64 blocks of >= 64 columns can
+// instead run on the tensor-core kernels of subst_tc.cu; the autotuner decides per batch signature.
 #include <algorithm>
 
 #include "hz_internal.cuh"
@@ -39,17 +48,21 @@ template <> __device__ inline void atomic_sub<double2>(double2* p, double2 v) {
 }
 template <class C> __device__ inline void atomic_add(C* p, C v) { atomic_sub(p, cneg(v)); }
 
+// Complex64 factors hold M21 (see above).
+template <class C> constexpr bool has_m21 = sizeof(C) == 8;
+
 // Writes the TILE x CC output block of one task, staged in shared memory (Ys, row pitch YP),
 // to the solve vectors: consecutive threads take consecutive columns of a row, and every thread
 // issues all of its loads (row indices, D^{-1}, z) before any of its writes.  A task covering
-// the whole reduction of its rows is their only writer and stores; split reductions and FB
-// (update rows are shared between the nodes of a level) accumulate atomically.  Outputs are
-// zeroed beforehand (x before the forward pass and, for BB, by BA; acc before the backward).
+// the whole reduction of its rows is their only writer and stores; split reductions and updates
+// of rows that hold a value already (FB, whose rows nodes of a level share; BA on M21) accumulate
+// atomically.  Stored outputs are zeroed beforehand.
 template <class C, int CC, int MODE>
 __device__ inline void write_out(const C* Ys, int YP, const JobDev<C>& jb, const NodeDev& nd, const int* upd,
                                  int tile, int col0, int ldc, int kt0, bool unique) {
     constexpr int EPT = (TILE * CC + 255) / 256;   // elements per thread
     constexpr int EB = EPT < 4 ? EPT : 4;          // elements per load batch
+    constexpr bool M21 = has_m21<C>;
     const int nrows = (MODE == FB) ? nd.nupd : nd.nown;
 #pragma unroll
     for (int i0 = 0; i0 < EPT; i0 += EB) {
@@ -69,7 +82,8 @@ __device__ inline void write_out(const C* Ys, int YP, const JobDev<C>& jb, const
             if (v[i]) {
                 dst[i] = ((MODE == FB) ? (long long)upd[row] : (long long)(nd.own0 + row)) * ldc + col0 + c;
                 y[i] = Ys[r * YP + c];
-                if (MODE == BA && kt0 == 0) {
+                if (M21 && MODE == FA) y[i] = cmul(jb.dinv[nd.own0 + row], y[i]);
+                if (!M21 && MODE == BA && kt0 == 0) {
                     di[i] = jb.dinv[nd.own0 + row];
                     z[i] = jb.x[dst[i]];
                 }
@@ -78,11 +92,12 @@ __device__ inline void write_out(const C* Ys, int YP, const JobDev<C>& jb, const
 #pragma unroll
         for (int i = 0; i < EB; ++i) {
             if (!v[i]) continue;
-            if (MODE == FB) {
+            if (MODE == FB || (M21 && MODE == BA)) {
                 atomic_sub(jb.acc + dst[i], y[i]);
             } else if (MODE == FA || MODE == BB) {
-                if (unique) jb.x[dst[i]] = y[i];
-                else atomic_add(jb.x + dst[i], y[i]);
+                C* out = (M21 && MODE == BB) ? jb.acc : jb.x;
+                if (unique) out[dst[i]] = y[i];
+                else atomic_add(out + dst[i], y[i]);
             } else {  // BA: acc = Dinv z - L21^T x_upd; the task with the first reduction tile clears z
                 C val = y[i];
                 if (kt0 == 0) {
@@ -94,6 +109,12 @@ __device__ inline void write_out(const C* Ys, int YP, const JobDev<C>& jb, const
             }
         }
     }
+}
+
+// the vector a product reads
+template <int MODE, class C> __device__ inline const C* source_vec(const JobDev<C>& jb) {
+    if (has_m21<C>) return MODE == BB ? jb.x : jb.acc;
+    return (MODE == FA || MODE == BB) ? jb.acc : jb.x;
 }
 
 template <class C, int CC, int MODE>
@@ -125,7 +146,7 @@ __global__ void __launch_bounds__(256) k_subst(const Task* __restrict__ tasks,
     const int kt0 = tk.pad_;
     const int kt1 = min(kend, kt0 + KS);
 
-    const C* vec = (MODE == FA || MODE == BB) ? jb.acc : jb.x;
+    const C* vec = source_vec<MODE>(jb);
     const int* upd = jb.upd_idx + nd.upd_off;
 
     C acc[NCT];
@@ -237,7 +258,7 @@ __global__ void __launch_bounds__(256, 4) k_subst64(const Task* __restrict__ tas
     else kend = nd.own_t;
     const int kt0 = tk.pad_;
     const int kt1 = min(kend, kt0 + KS);
-    const float2* vec = (MODE == FA || MODE == BB) ? jb.acc : jb.x;
+    const float2* vec = source_vec<MODE>(jb);
     const int* upd = jb.upd_idx + nd.upd_off;
 
     float2 acc[2][4];
@@ -341,12 +362,15 @@ void launch_level(const Batch& b, int h, int mode, int ldc, cudaStream_t st) {
     HZ_CHECK_LAUNCH();
 }
 
-template <class C>
-void zero_vectors(const Batch& b, bool x_vec, int ldc, cudaStream_t st) {
-    for (size_t j = 0; j < b.vec_ptrs.size(); ++j) {
-        void* p = x_vec ? b.vec_ptrs[j].second : b.vec_ptrs[j].first;
-        HZ_CUDA(cudaMemsetAsync(p, 0, (size_t)b.vec_rows[j] * ldc * sizeof(C), st));
-    }
+// One launch for the vectors of all layers (a memset node per layer costs a launch each: 2 x 16
+// of them per substitution at 16 layers).  16-byte stores, grid-stride; HBM/L2 write bound.
+__global__ void __launch_bounds__(256) k_zero(const ZeroDev* d) {
+    const ZeroDev z = d[blockIdx.y];
+    float4* p = (float4*)z.p;
+    const long long n16 = z.bytes / 16;
+    for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n16; i += (long long)gridDim.x * 256)
+        p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (blockIdx.x == 0 && threadIdx.x == 0 && (z.bytes & 8)) ((double*)z.p)[2 * n16] = 0.0;
 }
 
 // Records a CUDA event pair around one launch in profiling detail mode.
@@ -390,15 +414,36 @@ void run_batch(const Batch& b, int ldc, int ncols, bool tc, int* flag, cudaStrea
             lt.done();
         }
     };
-    zero_vectors<C>(b, true, ldc, st);
+    auto zero = [&](int which, int mode) {   // acc (0) / x (1) of every layer, before the launches of `mode`
+        LaunchTimer lt(pl, st, 0, 0.0, 0.0, mode, 0, (long long)b.vec_rows.size());
+        launch_zero(b.d_zero[which], (int)b.vec_rows.size(), b.zero_max, st);
+        lt.done();
+    };
+    if (has_m21<C>) {   // FA and BB hold the nodes of all levels at index 0
+        for (int h = 0; h < b.H; ++h) level(h, FB);
+        zero(1, FA);
+        level(0, FA);
+        zero(0, BB);
+        level(0, BB);
+        for (int h = b.H - 1; h >= 0; --h) level(h, BA);
+        return;
+    }
+    zero(1, FA);
     for (int h = 0; h < b.H; ++h)
         for (int mode : {FA, FB}) level(h, mode);
-    zero_vectors<C>(b, false, ldc, st);
+    zero(0, BA);
     for (int h = b.H - 1; h >= 0; --h)
         for (int mode : {BA, BB}) level(h, mode);
 }
 
 }  // namespace
+
+void launch_zero(const ZeroDev* d, int n, long long max_bytes, cudaStream_t st) {
+    if (n <= 0 || max_bytes <= 0) return;
+    const unsigned gx = (unsigned)std::max<long long>(1, std::min<long long>(cdiv(max_bytes / 16, 1024), 1216));
+    k_zero<<<dim3(gx, (unsigned)n), 256, 0, st>>>(d);
+    HZ_CHECK_LAUNCH();
+}
 
 int chunk_cols(bool is_double, int ncols) {
     const int cmax = is_double ? 32 : 64;
@@ -571,6 +616,7 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
     int H = 0;
     for (int l : layers) H = std::max(H, (int)ctx.shapes[ctx.layers[l].shape].levels.size());
     b.H = H;
+    const bool m21 = has_m21<C>;
     std::vector<std::vector<Task>> lists[4], quads[4];
     for (auto& v : lists) v.assign(H, {});
     for (auto& v : quads) v.assign(H, {});
@@ -620,25 +666,31 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
                     const int out_t = mode == 1 ? nd.upd_t : nd.own_t;
                     const bool on_tc = tc && tc_node(mode, nd, b.min_t);
                     int nact = 0;
+                    if (m21 && mode == 2 && nd.nupd == 0) continue;   // the root has nothing to gather
+                    // M21: FA and BB of every level go in one launch each
+                    const int hl = (m21 && (mode == 0 || mode == 3)) ? 0 : h;
                     for (int q = 0; q < nblk; ++q) {
-                        const bool on = fwd ? (fcode[q] == SP_ALL || touches(fplanes[q]))
-                                            : (bcode[q] == SP_ALL || touches(bplanes[q]));
+                        const bool fon = fcode[q] == SP_ALL || touches(fplanes[q]);
+                        const bool bon = bcode[q] == SP_ALL || touches(bplanes[q]);
+                        // on M21, FA and BB turn a node's right-hand side into its part of the
+                        // solution: both are needed only where the one is nonzero and the other read
+                        const bool on = (m21 && (mode == 0 || mode == 3)) ? fon && bon : (fwd ? fon : bon);
                         if (!on) continue;
                         ++nact;
                         const int jq = j * nblk + q;
                         if (on_tc) {
                             for (int t = 0; t < out_t; t += 4) {
-                                if (mode == 0) add_tasks(quads[0][h], jq, nid, t, 0, std::min(t + 4, nd.own_t), b.KS_tc);
-                                if (mode == 1) add_tasks(quads[1][h], jq, nid, t, 0, nd.own_t, b.KS_tc);
-                                if (mode == 2) add_tasks(quads[2][h], jq, nid, t, 0, nd.upd_t, b.KS_tc);
-                                if (mode == 3) add_tasks(quads[3][h], jq, nid, t, t, nd.own_t, b.KS_tc);
+                                if (mode == 0) add_tasks(quads[0][hl], jq, nid, t, 0, std::min(t + 4, nd.own_t), b.KS_tc);
+                                if (mode == 1) add_tasks(quads[1][hl], jq, nid, t, 0, nd.own_t, b.KS_tc);
+                                if (mode == 2) add_tasks(quads[2][hl], jq, nid, t, 0, nd.upd_t, b.KS_tc);
+                                if (mode == 3) add_tasks(quads[3][hl], jq, nid, t, t, nd.own_t, b.KS_tc);
                             }
                         } else {
                             for (int t = 0; t < out_t; ++t) {
-                                if (mode == 0) add_tasks(lists[0][h], jq, nid, t, 0, t + 1, KS);      // FA: Linv row tile t
-                                if (mode == 1) add_tasks(lists[1][h], jq, nid, t, 0, nd.own_t, KS);   // FB: L21 row tile t
-                                if (mode == 2) add_tasks(lists[2][h], jq, nid, t, 0, nd.upd_t, KS);   // BA (>= 1 task)
-                                if (mode == 3) add_tasks(lists[3][h], jq, nid, t, t, nd.own_t, KS);   // BB
+                                if (mode == 0) add_tasks(lists[0][hl], jq, nid, t, 0, t + 1, KS);      // FA: Linv row tile t
+                                if (mode == 1) add_tasks(lists[1][hl], jq, nid, t, 0, nd.own_t, KS);   // FB: L21 row tile t
+                                if (mode == 2) add_tasks(lists[2][hl], jq, nid, t, 0, nd.upd_t, KS);   // BA (>= 1 task)
+                                if (mode == 3) add_tasks(lists[3][hl], jq, nid, t, t, nd.own_t, KS);   // BB
                             }
                         }
                     }
@@ -647,22 +699,31 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
                     // algorithmically, however many column blocks use them
                     const double ent = (mode == FA || mode == BB) ? (double)nd.nown * (nd.nown + 1) / 2.0
                                                                   : (double)nd.nown * nd.nupd;
-                    b.lvl_bytes[on_tc][mode][h] += ent * sizeof(C);
-                    b.lvl_flops[on_tc][mode][h] += 8.0 * ent * nact / nblk;
+                    b.lvl_bytes[on_tc][mode][hl] += ent * sizeof(C);
+                    b.lvl_flops[on_tc][mode][hl] += 8.0 * ent * nact / nblk;
                 }
             }
     }
-    // tensor-core work items longest reduction first: the persistent kernel deals them out
-    // round-robin, and either kernel then ends a launch on short items
+    // work items longest reduction first: the persistent tensor-core kernel deals them out
+    // round-robin, and every kernel then ends a launch on short items
     for (int mode = 0; mode < 4; ++mode)
         for (int h = 0; h < H; ++h) {
-            auto red_len = [&](const Task& tk) {
-                const Node& nd = ctx.shapes[ctx.layers[layers[tk.job / nblk]].shape].nodes[tk.node];
-                const int kend = mode == 0 ? std::min(tk.tile + 4, nd.own_t) : (mode == 2 ? nd.upd_t : nd.own_t);
-                return std::min(kend, tk.pad_ + std::min(b.KS_tc, 1 << 28)) - tk.pad_;
+            auto sort_items = [&](std::vector<Task>& v, int rows, int ks) {
+                auto red_len = [&](const Task& tk) {
+                    const Node& nd = ctx.shapes[ctx.layers[layers[tk.job / nblk]].shape].nodes[tk.node];
+                    const int kend = mode == 0 ? std::min(tk.tile + rows, nd.own_t) : (mode == 2 ? nd.upd_t : nd.own_t);
+                    return std::min(kend, tk.pad_ + std::min(ks, 1 << 28)) - tk.pad_;
+                };
+                std::vector<std::pair<int, int>> order(v.size());
+                for (int i = 0; i < (int)v.size(); ++i) order[i] = {-red_len(v[i]), i};
+                std::sort(order.begin(), order.end());
+                std::vector<Task> sorted;
+                sorted.reserve(v.size());
+                for (auto& o : order) sorted.push_back(v[o.second]);
+                v.swap(sorted);
             };
-            std::stable_sort(quads[mode][h].begin(), quads[mode][h].end(),
-                             [&](const Task& x, const Task& y) { return red_len(x) > red_len(y); });
+            sort_items(quads[mode][h], 4, b.KS_tc);
+            if (m21) sort_items(lists[mode][h], 1, KS);
         }
     std::vector<Task> all;
     for (int mode = 0; mode < 4; ++mode) {
@@ -711,6 +772,17 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
                 b.alg_bytes += b.lvl_bytes[k][mode][h];
                 b.flops_per_col += b.lvl_flops[k][mode][h];
             }
+    for (int w = 0; w < 2; ++w) {
+        std::vector<ZeroDev> zd;
+        for (size_t j = 0; j < b.vec_ptrs.size(); ++j) {
+            const long long bytes = b.vec_rows[j] * ldc * (long long)sizeof(C);
+            zd.push_back({w ? b.vec_ptrs[j].second : b.vec_ptrs[j].first, bytes});
+            b.zero_max = std::max(b.zero_max, bytes);
+        }
+        HZ_CUDA(cudaMalloc(&b.d_zero[w], zd.size() * sizeof(ZeroDev)));
+        HZ_CUDA(cudaMemcpyAsync(b.d_zero[w], zd.data(), zd.size() * sizeof(ZeroDev), cudaMemcpyHostToDevice, ctx.stream));
+        HZ_CUDA(cudaStreamSynchronize(ctx.stream));
+    }
     HZ_CUDA(cudaMalloc(&b.d_jobs, jobs.size() * sizeof(JobDev<C>)));
     HZ_CUDA(cudaMemcpyAsync(b.d_jobs, jobs.data(), jobs.size() * sizeof(JobDev<C>), cudaMemcpyHostToDevice,
                             ctx.stream));
@@ -722,6 +794,8 @@ void free_batches(Ctx& ctx) {
     for (auto& kv : ctx.batches) {
         cudaFree(kv.second.d_tasks);
         cudaFree(kv.second.d_jobs);
+        cudaFree(kv.second.d_zero[0]);
+        cudaFree(kv.second.d_zero[1]);
     }
     ctx.batches.clear();
 }

@@ -33,7 +33,7 @@
 //               MMA warp accumulates item i+1, so block start-up, pipeline fill and epilogue are
 //               paid once per SM instead of once per item.
 // Output rule of both: an item that covers the full reduction of its rows stores them; split
-// reductions and the shared update rows of FB accumulate with vector atomics.  Every mbarrier
+// reductions and the updates (FB, BA) accumulate with vector atomics.  Every mbarrier
 // wait is bounded (polls and wall time); a wait that gives up raises an abort flag in shared
 // memory that ends the block's other waits; the block then records an error flag, waits
 // (bounded) for its own MMAs, frees its tensor memory and exits.
@@ -89,7 +89,7 @@ __device__ inline Item decode(const Task* tasks, const JobDev<float2>* jobs, lon
     const int kfull1 = (MODE == FA) ? min(it.o0 + 4, nd.own_t) : ((MODE == BA) ? nd.upd_t : nd.own_t);
     it.kend = min(kfull1, it.kbeg + KS);
     it.nst = max(0, it.kend - it.kbeg) * 2;
-    it.unique = it.kbeg == kfull0 && it.kend == kfull1 && MODE != FB;
+    it.unique = it.kbeg == kfull0 && it.kend == kfull1 && MODE != FB && MODE != BA;
     return it;
 }
 
@@ -146,7 +146,7 @@ __device__ inline void load_stage(unsigned char* rb, const Item& it, int s, int 
         }
         cp16(dst, exists ? (const void*)src : (const void*)it.jb.fac, exists ? 16 : 0);
     }
-    const float2* vec = (MODE == FA || MODE == BB) ? it.jb.acc : it.jb.x;
+    const float2* vec = MODE == BB ? it.jb.x : it.jb.acc;
 #pragma unroll
     for (int i = 0; i < KC * NT / 2 / NLOAD; ++i) {  // vector rows: KC x NT, raw [k][n]
         const int c = t + NLOAD * i;
@@ -206,25 +206,18 @@ __device__ inline void convert_stage(const unsigned char* rb, unsigned char* cv,
     }
 }
 
-// Writes one 16-byte column pair y of an output row (global offset base + c) by the output rule.
+// Writes one 16-byte column pair y of an output row (global offset base + c) by the output rule;
+// d is the row's D^{-1} (FA).
 template <int MODE>
-__device__ inline void write_pair(const Item& it, long long base, int c, float4 y, float2 d, float4 z) {
-    float4* dx = (float4*)(it.jb.x + base + c);
-    float4* da = (float4*)(it.jb.acc + base + c);
-    if (MODE == FB) {
-        atomicAdd(da, make_float4(-y.x, -y.y, -y.z, -y.w));
-    } else if (MODE == FA || MODE == BB) {
-        if (it.unique) *dx = y;
-        else atomicAdd(dx, y);
-    } else {  // BA: acc = Dinv z - partial; the first split clears z
-        if (it.kbeg == 0) {
-            y.x -= d.x * z.x - d.y * z.y; y.y -= d.x * z.y + d.y * z.x;
-            y.z -= d.x * z.z - d.y * z.w; y.w -= d.x * z.w + d.y * z.z;
-            *dx = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        const float4 ny = make_float4(-y.x, -y.y, -y.z, -y.w);
-        if (it.unique) *da = ny;
-        else atomicAdd(da, ny);
+__device__ inline void write_pair(const Item& it, long long base, int c, float4 y, float2 d) {
+    if (MODE == FB || MODE == BA) {
+        atomicAdd((float4*)(it.jb.acc + base + c), make_float4(-y.x, -y.y, -y.z, -y.w));
+    } else {
+        if (MODE == FA)
+            y = make_float4(d.x * y.x - d.y * y.y, d.x * y.y + d.y * y.x, d.x * y.z - d.y * y.w, d.x * y.w + d.y * y.z);
+        float4* dst = (float4*)((MODE == FA ? it.jb.x : it.jb.acc) + base + c);
+        if (it.unique) *dst = y;
+        else atomicAdd(dst, y);
     }
 }
 
@@ -312,7 +305,7 @@ k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jo
         for (int r = t; r < MR; r += NLOAD) {
             const long long base = row_base<MODE>(it, r, ldc);
             rowbase[r] = base;
-            if (MODE == BA) dinv_s[r] = base >= 0 ? it.jb.dinv[it.nd.own0 + it.o0 * TILE + r] : make_float2(0.f, 0.f);
+            if (MODE == FA) dinv_s[r] = base >= 0 ? it.jb.dinv[it.nd.own0 + it.o0 * TILE + r] : make_float2(0.f, 0.f);
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
     } else if (t < NLOAD + NCONV) {
@@ -358,15 +351,13 @@ k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jo
     // ---- epilogue (converter warps), per column half of the tile:
     //  (1) tensor memory -> shared staging tile [128 rows][HALF + 2]; warp w may read TMEM lanes
     //      32 (w % 4) .. +31 (output tile o0 + w % 4); the two warps of a lane quarter split the columns;
-    //  (2) each converter warp writes 16 staged rows, lane = pair of columns (16-byte accesses),
-    //      all loads of a batch of rows (BA's z) before its writes.
+    //  (2) each converter warp writes 16 staged rows, lane = pair of columns (16-byte accesses).
     if (ok && t >= NLOAD && t < NLOAD + NCONV) {
         constexpr int HALF = LY::HALF, SP = LY::SP;
         constexpr int CPW = HALF / 2;            // columns per warp per pass
         constexpr int RPW = MR / (NCONV / 32);   // staged rows written per warp
         constexpr int NP = HALF / 2;             // 16-byte column pairs per row and pass
-        constexpr int RB = 8;                    // rows per load batch
-        static_assert(CPW % 16 == 0 && RPW % RB == 0, "epilogue tiling");
+        static_assert(CPW % 16 == 0, "epilogue tiling");
         float2* stg = (float2*)smem;             // operand and raw buffers are free after the MMAs
         const int cw = (t - NLOAD) >> 5;
         const int q4 = w & 3, sub = cw >> 2;
@@ -391,22 +382,13 @@ k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jo
             asm volatile("bar.sync 1, %0;" :: "n"(NCONV) : "memory");   // converter warps only
             const bool lane_on = l < NP;
             const int c = pass * HALF + 2 * l;
-            for (int i0 = 0; i0 < RPW; i0 += RB) {
-                float4 z[RB];
-#pragma unroll
-                for (int r = 0; r < RB; ++r) {
-                    z[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    const long long base = rowbase[cw * RPW + i0 + r];
-                    if (MODE == BA && it.kbeg == 0 && lane_on && base >= 0) z[r] = *(const float4*)(it.jb.x + base + c);
-                }
-#pragma unroll
-                for (int r = 0; r < RB; ++r) {
-                    const int rl2 = cw * RPW + i0 + r;
-                    const long long base = rowbase[rl2];
-                    if (!lane_on || base < 0) continue;
-                    const float2 d = (MODE == BA) ? dinv_s[rl2] : make_float2(0.f, 0.f);
-                    write_pair<MODE>(it, base, c, *(const float4*)&stg[rl2 * SP + 2 * l], d, z[r]);
-                }
+#pragma unroll 8
+            for (int i = 0; i < RPW; ++i) {
+                const int rl2 = cw * RPW + i;
+                const long long base = rowbase[rl2];
+                if (!lane_on || base < 0) continue;
+                const float2 d = (MODE == FA) ? dinv_s[rl2] : make_float2(0.f, 0.f);
+                write_pair<MODE>(it, base, c, *(const float4*)&stg[rl2 * SP + 2 * l], d);
             }
             asm volatile("bar.sync 1, %0;" :: "n"(NCONV) : "memory");   // staging reused by the next pass
         }
@@ -574,7 +556,7 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
             // this lane's row descriptor, shuffled to the writing lanes below
             const long long my_base = row_base<MODE>(it, 32 * q4 + l, ldc);
             float2 my_d = make_float2(0.f, 0.f);
-            if (MODE == BA && my_base >= 0) my_d = it.jb.dinv[it.nd.own0 + it.o0 * TILE + 32 * q4 + l];
+            if (MODE == FA && my_base >= 0) my_d = it.jb.dinv[it.nd.own0 + it.o0 * TILE + 32 * q4 + l];
             ok = mbar_wait(smem_u32(acc_full + b), (uint32_t)((nit >> 1) & 1), abort, polls);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -595,22 +577,17 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
                                                                  __uint_as_float(vr[j + 1]), __uint_as_float(vi[j + 1]));
                 __syncwarp();
                 const int c = c0 + 2 * p;
-                long long base[8];
-                float4 z[8];
-#pragma unroll
-                for (int g = 0; g < 8; ++g) {   // all loads of the chunk before its writes
-                    base[g] = __shfl_sync(0xffffffffu, my_base, 4 * g + r4);
-                    z[g] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (MODE == BA && it.kbeg == 0 && base[g] >= 0) z[g] = *(const float4*)(it.jb.x + base[g] + c);
-                }
 #pragma unroll
                 for (int g = 0; g < 8; ++g) {
                     const int rr = 4 * g + r4;
-                    float2 d;
-                    d.x = __shfl_sync(0xffffffffu, my_d.x, rr);
-                    d.y = __shfl_sync(0xffffffffu, my_d.y, rr);
-                    if (base[g] < 0) continue;
-                    write_pair<MODE>(it, base[g], c, *(const float4*)&stg[rr * LY::EP + 2 * p], d, z[g]);
+                    const long long base = __shfl_sync(0xffffffffu, my_base, rr);
+                    float2 d = make_float2(0.f, 0.f);
+                    if (MODE == FA) {
+                        d.x = __shfl_sync(0xffffffffu, my_d.x, rr);
+                        d.y = __shfl_sync(0xffffffffu, my_d.y, rr);
+                    }
+                    if (base < 0) continue;
+                    write_pair<MODE>(it, base, c, *(const float4*)&stg[rr * LY::EP + 2 * p], d);
                 }
                 __syncwarp();
             }

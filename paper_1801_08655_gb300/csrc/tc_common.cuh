@@ -113,8 +113,12 @@ __device__ __forceinline__ void tmem_ld16(uint32_t ar, uint32_t ai, uint32_t (&v
 // MMA part of a stage (one thread): 2 x (4 or 12) MMAs of 8 complex reduction indices.  The
 // converted operands of a stage sit at `base`: Ar_hi, Ar_lo, Ai_hi, Ai_lo (MR x KC each), then
 // Xr_hi, Xr_lo, Xi_hi, Xi_lo (NT x KC each); the product is Y[MR x NT] = A X^T.
-template <int NT, int SPLIT>
+// SEP: the hi x lo and lo x hi terms go to accumulators of their own, 2 NT columns after tm_r and
+// tm_i, to be added by the reader: the tensor core truncates at every accumulation, so a third of
+// the accumulations into the large sum is a third of its error (at the same MMAs).
+template <int NT, int SPLIT, bool SEP = false>
 __device__ __forceinline__ void mma_stage(uint32_t base, uint32_t tm_r, uint32_t tm_i, bool first_stage) {
+    const uint32_t tl_r = SEP ? tm_r + 2 * NT : tm_r, tl_i = SEP ? tm_i + 2 * NT : tm_i;
     constexpr int A_MAT = MR * KC * 4, X_MAT = NT * KC * 4;   // one real operand matrix of A / of X
     const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(NT >> 3) << 17) | ((uint32_t)(MR >> 4) << 24);
     const uint32_t idesc_neg = idesc | (1u << 13);
@@ -132,14 +136,14 @@ __device__ __forceinline__ void mma_stage(uint32_t base, uint32_t tm_r, uint32_t
         mma_tf32(tm_i, aih, xrh, idesc, first);      // Yi = Ai Xr + Ar Xi
         mma_tf32(tm_i, arh, xih, idesc, 1u);
         if (SPLIT == 3) {                             // hi x lo and lo x hi terms
-            mma_tf32(tm_r, arh, xrl, idesc, 1u);
-            mma_tf32(tm_r, arl, xrh, idesc, 1u);
-            mma_tf32(tm_r, aih, xil, idesc_neg, 1u);
-            mma_tf32(tm_r, ail, xih, idesc_neg, 1u);
-            mma_tf32(tm_i, aih, xrl, idesc, 1u);
-            mma_tf32(tm_i, ail, xrh, idesc, 1u);
-            mma_tf32(tm_i, arh, xil, idesc, 1u);
-            mma_tf32(tm_i, arl, xih, idesc, 1u);
+            mma_tf32(tl_r, arh, xrl, idesc, SEP ? first : 1u);
+            mma_tf32(tl_r, arl, xrh, idesc, 1u);
+            mma_tf32(tl_r, aih, xil, idesc_neg, 1u);
+            mma_tf32(tl_r, ail, xih, idesc_neg, 1u);
+            mma_tf32(tl_i, aih, xrl, idesc, SEP ? first : 1u);
+            mma_tf32(tl_i, ail, xrh, idesc, 1u);
+            mma_tf32(tl_i, arh, xil, idesc, 1u);
+            mma_tf32(tl_i, arl, xih, idesc, 1u);
         }
     }
 }
