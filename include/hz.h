@@ -110,7 +110,7 @@ void hz_default_opts(hz_precision prec, hz_solve_opts* opts);
  * Errors: HZ_ERR_ARG, HZ_ERR_NONFINITE (m), HZ_ERR_OOM, HZ_ERR_CUDA.
  * Environment variables read here (they change speed, never the solution beyond rounding):
  *   HZ_SUBST_TC       complex64 substitutions on the tcgen05 kernel: 0 never, 1 always (for
- *                     column blocks of >= 64), 2 (default) when the autotuner times it faster
+ *                     more than 16 columns), 2 (default) when the autotuner times it faster
  *   HZ_TC_MIN_TILES   default minimum output tiles of a tensor-core product (8)
  *   HZ_PRECOND_SPLIT  1: single-term TF32 tensor-core products inside the preconditioner
  *                     (default 3 terms, FP32-level)

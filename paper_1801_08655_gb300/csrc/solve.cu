@@ -22,7 +22,7 @@
 // few nodes with long reductions, spread over the whole GPU).  Stored outputs are zeroed
 // beforehand; a task covering the whole reduction of its rows stores them, split reductions and
 // the updates (FB, complex64 BA) accumulate with atomics.  The factor tile stream is the HBM
-// traffic that bounds the kernel at small column counts.  Complex64 blocks of >= 64 columns can
+// traffic that bounds the kernel at small column counts.  Complex64 blocks of more than 16 columns can
 // instead run on the tensor-core kernels of subst_tc.cu; the autotuner decides per batch signature.
 #include <algorithm>
 
@@ -499,6 +499,15 @@ static bool tc_node(int mode, const Node& nd, int min_tiles) {
     return out_t >= min_tiles && red_t >= (min_tiles <= 2 ? 1 : 2);
 }
 
+// Tensor-core column tiles exist for this leading dimension.  32-column blocks stay on the CUDA cores
+// when the factors come from FP64: the products' own rounding (about 2e-6 of a 40^3 layer solve on
+// the tensor cores, 2e-7 here) is then the larger part of a local solve's error; with complex64
+// factors (1e-5) it is not.
+static bool tc_usable(const Ctx& ctx, int ldc) {
+    const int nt = tc_columns(ldc);
+    return nt > 32 || (nt == 32 && ctx.prec == HZ_PREC_MIXED);
+}
+
 static std::string tune_key(const Ctx& ctx, const std::vector<int>& layers, int ldc, int split, int sparse) {
     std::vector<int> shapes;
     for (int l : layers) shapes.push_back(ctx.layers[l].shape);
@@ -512,7 +521,7 @@ template <class C>
 Batch& get_batch(Ctx& ctx, const std::vector<int>& layers, int ncols, int split, int sparse) {
     const bool dbl = sizeof(C) == 16;
     const int ldc = padded_ldc(dbl, ncols);
-    const bool tc_ok = !dbl && tc_columns(ldc) > 0;
+    const bool tc_ok = !dbl && tc_usable(ctx, ldc);
     auto it = ctx.tuned.find(tune_key(ctx, layers, ldc, split, sparse));
     if (it != ctx.tuned.end()) {
         const auto& ch = it->second;
@@ -532,7 +541,7 @@ template <class C>
 void ensure_tuned(Ctx& ctx, const std::vector<int>& layers, int ncols, int split, int sparse) {
     const bool dbl = sizeof(C) == 16;
     const int ldc = padded_ldc(dbl, ncols);
-    const bool tc_ok = !dbl && tc_columns(ldc) > 0;
+    const bool tc_ok = !dbl && tc_usable(ctx, ldc);
     const std::string key = tune_key(ctx, layers, ldc, split, sparse);
     if (!ctx.autotune || ctx.tuned.count(key)) return;
     const int cc0 = chunk_cols(dbl, ncols);
@@ -546,10 +555,17 @@ void ensure_tuned(Ctx& ctx, const std::vector<int>& layers, int ncols, int split
             for (int ks : {4, 8, 16, 1 << 30})
                 if (!try_tc || ks == 8 || ks == (1 << 30)) cands.push_back({ks, cc, 0, 1 << 30, 0, 0});
     }
-    if (try_tc)
-        for (int cfg : {1, 0})   // persistent / one block per work item
-            for (int mt : {2, 4, ctx.tc_min_tiles})
-                for (int kstc : {16, 1 << 30}) cands.push_back({8, cc0, 1, kstc, mt, cfg});
+    if (try_tc) {
+        // every product of two output tiles or more (fewer never won); persistent kernel at all
+        // depths (a single layer's steps want 2-8 tiles a work item, 64^3 with 128 columns: 0.62 ms
+        // at 4 against 0.88 at 16; all layers together 16 and more), one block per item at two
+        std::vector<int> mts{2};
+        if (ctx.tc_min_tiles < 8 && ctx.tc_min_tiles != 2) mts.push_back(ctx.tc_min_tiles);
+        for (int mt : mts) {
+            for (int kstc : {2, 4, 8, 16, 1 << 30}) cands.push_back({8, cc0, 1, kstc, mt, 1});
+            for (int kstc : {4, 1 << 30}) cands.push_back({8, cc0, 1, kstc, mt, 0});
+        }
+    }
     cudaEvent_t e0, e1;
     HZ_CUDA(cudaEventCreate(&e0));
     HZ_CUDA(cudaEventCreate(&e1));

@@ -1,7 +1,7 @@
 // Tensor-core (tcgen05) variant of the substitution products for complex64 factors.
 //
-// A work item computes 128 complex output rows (four factor tile rows) x NT right-hand-side
-// columns of one of the four node products of the substitution (see solve.cu), for the nodes
+// A work item computes 128 complex output rows (four factor tile rows) x NT = 32, 64 or 128
+// right-hand-side columns of one of the four node products of the substitution (see solve.cu), for the nodes
 // whose products are large enough to fill it; smaller nodes of the same tree level run on the
 // CUDA-core kernel in the same phase.
 //
@@ -52,16 +52,51 @@ using namespace tcc;
 
 enum { FA = 0, FB = 1, BA = 2, BB = 3 };
 
-// Sizes of one ring stage for NT columns.
+// Sizes of one ring stage for NT columns.  NT <= 64 runs the wide form of the MMAs (the output's
+// two halves side by side, three vector blocks per term); NT = 128 would need 6 x 8 KB of vector
+// operands per stage, which does not fit beside a two-deep raw ring, and fills N = 128 as it is.
+// The room that narrow tiles leave goes to the raw ring: the factor stream, 16 KB per stage
+// whatever NT is, binds them, and every further stage in flight covers memory latency.
+// Measured: a 32-column block of a 128^3 layer 3.10 ms on the CUDA cores, 1.68 here (115-120
+// TFLOP/s on the upper levels; about 1200 shared-memory cycles a stage allow 140); 64 columns, 64^3,
+// 8 layers: 3.98 ms with N = 64 MMAs on a two-deep ring, 2.80 in the wide form.
 template <int NT> struct Ring {
+    static constexpr bool WIDE = NT <= 64;
     static constexpr int A_MAT = MR * KC * 4;            // one real operand matrix (8 KB)
     static constexpr int X_MAT = NT * KC * 4;
-    static constexpr int CONV = 4 * A_MAT + 4 * X_MAT;   // Ar_h Ar_l Ai_h Ai_l  Xr_h Xr_l Xi_h Xi_l
+    // Ar_h Ar_l Ai_h Ai_l, then Xr_h Xr_l Xi_h Xi_l, or (WIDE) -Xi_h Xr_h Xi_h -Xi_l Xr_l Xi_l
+    static constexpr int CONV = 4 * A_MAT + (WIDE ? 6 : 4) * X_MAT;
     static constexpr int RAW_A = 4 * 32 * TROW;          // large enough for both raw tile layouts
     static constexpr int RAW_X = KC * NT * 8;
     static constexpr int RAW = RAW_A + RAW_X;
-    static constexpr int BYTES = 2 * (CONV + RAW);       // two-deep rings
+    static constexpr int RD = NT == 32 ? 4 : (NT == 64 ? 3 : 2);   // raw ring depth
+    static constexpr int BYTES = 2 * CONV + RD * RAW;    // converted operands: two-deep
 };
+
+// Columns of one accumulator set: real and imaginary part, and (SEP) the hi x lo terms' own.
+template <int NT, int SPLIT, bool SEP> constexpr int acc_cols = (SEP && SPLIT == 3) ? 4 * NT : 2 * NT;
+
+template <int NT, int SPLIT, bool SEP>
+__device__ __forceinline__ void mma_item_stage(uint32_t conv, uint32_t tm, bool first) {
+    static_assert(!Ring<NT>::WIDE || SEP, "the wide form keeps the hi x lo terms apart");
+    if constexpr (Ring<NT>::WIDE) mma_stage_wide<NT, SPLIT>(conv, tm, first);
+    else mma_stage<NT, SPLIT, SEP>(conv, tm, tm + NT, first);
+}
+
+// 16 accumulator columns from c0 on of this warp's lanes, the terms added up.
+template <int NT, int SPLIT, bool SEP>
+__device__ __forceinline__ void read_acc(uint32_t tm, int c0, uint32_t (&vr)[16], uint32_t (&vi)[16]) {
+    tmem_ld16(tm + (uint32_t)c0, tm + (uint32_t)(NT + c0), vr, vi);
+    if constexpr (SEP && SPLIT == 3) {
+        uint32_t lr[16], li[16];
+        tmem_ld16(tm + (uint32_t)(2 * NT + c0), tm + (uint32_t)(3 * NT + c0), lr, li);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            vr[j] = __float_as_uint(__uint_as_float(vr[j]) + __uint_as_float(lr[j]));
+            vi[j] = __float_as_uint(__uint_as_float(vi[j]) + __uint_as_float(li[j]));
+        }
+    }
+}
 
 // One work item: 128 output rows (tiles o0 .. o0+3) x NT columns of one node product, reduction
 // tiles [kbeg, kend).
@@ -197,11 +232,24 @@ __device__ inline void convert_stage(const unsigned char* rb, unsigned char* cv,
         rh.x = tf32_hi(re[0]); rh.y = tf32_hi(re[1]); rh.z = tf32_hi(re[2]); rh.w = tf32_hi(re[3]);
         ih.x = tf32_hi(im[0]); ih.y = tf32_hi(im[1]); ih.z = tf32_hi(im[2]); ih.w = tf32_hi(im[3]);
         const int off = 4 * RG::A_MAT + coff(n, 4 * kq);
-        *(float4*)(cv + off + 0 * RG::X_MAT) = rh;
-        *(float4*)(cv + off + 2 * RG::X_MAT) = ih;
-        if (SPLIT == 3) {
-            *(float4*)(cv + off + 1 * RG::X_MAT) = make_float4(re[0] - rh.x, re[1] - rh.y, re[2] - rh.z, re[3] - rh.w);
-            *(float4*)(cv + off + 3 * RG::X_MAT) = make_float4(im[0] - ih.x, im[1] - ih.y, im[2] - ih.z, im[3] - ih.w);
+        const float4 rl = make_float4(re[0] - rh.x, re[1] - rh.y, re[2] - rh.z, re[3] - rh.w);
+        const float4 il = make_float4(im[0] - ih.x, im[1] - ih.y, im[2] - ih.z, im[3] - ih.w);
+        if (RG::WIDE) {
+            *(float4*)(cv + off + 0 * RG::X_MAT) = make_float4(-ih.x, -ih.y, -ih.z, -ih.w);
+            *(float4*)(cv + off + 1 * RG::X_MAT) = rh;
+            *(float4*)(cv + off + 2 * RG::X_MAT) = ih;
+            if (SPLIT == 3) {
+                *(float4*)(cv + off + 3 * RG::X_MAT) = make_float4(-il.x, -il.y, -il.z, -il.w);
+                *(float4*)(cv + off + 4 * RG::X_MAT) = rl;
+                *(float4*)(cv + off + 5 * RG::X_MAT) = il;
+            }
+        } else {
+            *(float4*)(cv + off + 0 * RG::X_MAT) = rh;
+            *(float4*)(cv + off + 2 * RG::X_MAT) = ih;
+            if (SPLIT == 3) {
+                *(float4*)(cv + off + 1 * RG::X_MAT) = rl;
+                *(float4*)(cv + off + 3 * RG::X_MAT) = il;
+            }
         }
     }
 }
@@ -236,12 +284,12 @@ __device__ inline long long row_base(const Item& it, int r, int ldc) {
 template <int NT> struct OneLayout {
     using RG = Ring<NT>;
     static constexpr int NTHREADS = NLOAD + NCONV + 32;
-    static constexpr int HALF = NT / 2;                  // output columns staged per epilogue pass
+    static constexpr int HALF = NT >= 64 ? NT / 2 : NT;  // output columns staged per epilogue pass
     static constexpr int SP = HALF + 2;                  // staging pitch (complex): 16-byte rows, odd in 16 B
     static_assert(MR * SP * 8 <= RG::BYTES, "staging tile must fit in the ring buffers");
     static constexpr int ROWS_OFF = RG::BYTES;           // long long rowbase[128], float2 dinv[128]
     static constexpr int BAR_OFF = ROWS_OFF + MR * 8 + MR * 8;
-    static constexpr int TOTAL = BAR_OFF + 8 * 8 + 16;
+    static constexpr int TOTAL = BAR_OFF + (2 * RG::RD + 4) * 8 + 16;
 };
 
 template <int NT, int MODE, int SPLIT>
@@ -252,17 +300,18 @@ k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jo
     using LY = OneLayout<NT>;
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char* conv = smem;                  // [2][CONV]
-    unsigned char* raw = smem + 2 * RG::CONV;    // [2][RAW]
+    unsigned char* raw = smem + 2 * RG::CONV;    // [RD][RAW]
+    constexpr int RD = RG::RD;
+    constexpr int TCOLS = acc_cols<NT, SPLIT, true>;
     long long* rowbase = (long long*)(smem + LY::ROWS_OFF);
     float2* dinv_s = (float2*)(smem + LY::ROWS_OFF + MR * 8);
-    uint64_t* bars = (uint64_t*)(smem + LY::BAR_OFF);
-    uint64_t* raw_full = bars;        // [2] loaders' copies landed (count NLOAD)
-    uint64_t* raw_empty = bars + 2;   // [2] converters done reading (count NCONV)
-    uint64_t* conv_full = bars + 4;   // [2] converted operands written (count NCONV)
-    uint64_t* conv_empty = bars + 6;  // [2] MMAs of the buffer done (tcgen05.commit)
-    uint32_t* tptr = (uint32_t*)(bars + 8);
-    volatile int* abort = (volatile int*)(bars + 8) + 1;
-    volatile int* committed = (volatile int*)(bars + 8) + 2;   // stages whose MMAs were committed
+    uint64_t* raw_full = (uint64_t*)(smem + LY::BAR_OFF);   // [RD] loaders' copies landed (count NLOAD)
+    uint64_t* raw_empty = raw_full + RD;   // [RD] converters done reading (count NCONV)
+    uint64_t* conv_full = raw_empty + RD;  // [2] converted operands written (count NCONV)
+    uint64_t* conv_empty = conv_full + 2;  // [2] MMAs of the buffer done (tcgen05.commit)
+    uint32_t* tptr = (uint32_t*)(conv_empty + 2);
+    volatile int* abort = (volatile int*)tptr + 1;
+    volatile int* committed = (volatile int*)tptr + 2;   // stages whose MMAs were committed
 
     const Item it = decode<NT, MODE>(tasks, jobs, blockIdx.x, nchunks, KS);
     const int t = threadIdx.x, w = t >> 5, l = t & 31;
@@ -270,13 +319,15 @@ k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jo
     const int mma_warp = (NLOAD + NCONV) / 32;
 
     if (w == mma_warp) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(tptr)), "r"(2 * NT));
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(tptr)), "r"(TCOLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (t == 0) {
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < RD; ++b) {
             mbar_init(raw_full + b, NLOAD);
             mbar_init(raw_empty + b, NCONV);
+        }
+        for (int b = 0; b < 2; ++b) {
             mbar_init(conv_full + b, NCONV);
             mbar_init(conv_empty + b, 1);
         }
@@ -287,15 +338,14 @@ k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jo
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tptr;
-    const uint32_t tm_r = tmem, tm_i = tmem + NT;  // accumulators: real part cols [0, NT), imag [NT, 2NT)
     bool ok = true;
 
     if (t < NLOAD) {
         Vrows<NT> rows = stage_rows<NT, MODE>(it, 0, t);
         for (int s = 0; s < nst && ok; ++s) {
-            const int slot = s & 1, use = s >> 1;
+            const int slot = s % RD, use = s / RD;
             const Vrows<NT> next = stage_rows<NT, MODE>(it, s + 1, t);   // looked up ahead
-            if (s >= 2) ok = mbar_wait(smem_u32(raw_empty + slot), (uint32_t)((use - 1) & 1), abort, polls);
+            if (s >= RD) ok = mbar_wait(smem_u32(raw_empty + slot), (uint32_t)((use - 1) & 1), abort, polls);
             if (!ok) break;
             load_stage<NT, MODE>(raw + slot * RG::RAW, it, s, ldc, t, rows);
             cp_async_arrive(raw_full + slot);
@@ -311,14 +361,14 @@ k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jo
     } else if (t < NLOAD + NCONV) {
         const int ct = t - NLOAD;
         for (int s = 0; s < nst && ok; ++s) {
-            const int slot = s & 1, use = s >> 1;
+            const int slot = s % RD, use = s / RD, cb = s & 1, cuse = s >> 1;
             ok = mbar_wait(smem_u32(raw_full + slot), (uint32_t)(use & 1), abort, polls);
-            if (ok && s >= 2) ok = mbar_wait(smem_u32(conv_empty + slot), (uint32_t)((use - 1) & 1), abort, polls);
+            if (ok && s >= 2) ok = mbar_wait(smem_u32(conv_empty + cb), (uint32_t)((cuse - 1) & 1), abort, polls);
             if (!ok) break;
-            convert_stage<NT, MODE, SPLIT>(raw + slot * RG::RAW, conv + slot * RG::CONV, ct);
+            convert_stage<NT, MODE, SPLIT>(raw + slot * RG::RAW, conv + cb * RG::CONV, ct);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_arrive(raw_empty + slot);
-            mbar_arrive(conv_full + slot);
+            mbar_arrive(conv_full + cb);
         }
     } else if (l == 0) {
         for (int s = 0; s < nst && ok; ++s) {
@@ -326,7 +376,7 @@ k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jo
             ok = mbar_wait(smem_u32(conv_full + cb), (uint32_t)(use & 1), abort, polls);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            mma_stage<NT, SPLIT>(smem_u32(conv + cb * RG::CONV), tm_r, tm_i, s == 0);
+            mma_item_stage<NT, SPLIT, true>(smem_u32(conv + cb * RG::CONV), tmem, s == 0);
             mma_commit(conv_empty + cb);
             *committed = s + 1;
         }
@@ -362,13 +412,13 @@ k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jo
         const int cw = (t - NLOAD) >> 5;
         const int q4 = w & 3, sub = cw >> 2;
         const int rl = 32 * q4 + l;
-        for (int pass = 0; pass < 2; ++pass) {
+        for (int pass = 0; pass < NT / HALF; ++pass) {
             const int cbeg = pass * HALF + sub * CPW;
             for (int c0 = cbeg; c0 < cbeg + CPW; c0 += 16) {
                 uint32_t vr[16], vi[16];
                 if (nst > 0) {
                     const uint32_t lane_off = (uint32_t)(32 * q4) << 16;
-                    tmem_ld16(tm_r + lane_off + (uint32_t)c0, tm_i + lane_off + (uint32_t)c0, vr, vi);
+                    read_acc<NT, SPLIT, true>(tmem + lane_off, c0, vr, vi);
                 } else {
 #pragma unroll
                     for (int j = 0; j < 16; ++j) { vr[j] = 0u; vi[j] = 0u; }
@@ -395,7 +445,7 @@ k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jo
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (w == mma_warp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(2 * NT));
+    if (w == mma_warp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(TCOLS));
 }
 
 // ------------------------------------------------------------------------------------------
@@ -408,8 +458,10 @@ template <int NT> struct PLayout {
     static constexpr int EP = 18;                          // staging pitch (complex) of a 32 x 16 chunk
     static constexpr int STG_OFF = RG::BYTES;              // 4 warps x 32 rows x EP complex
     static constexpr int BAR_OFF = STG_OFF + 4 * 32 * EP * 8;
-    static constexpr int TOTAL = BAR_OFF + 12 * 8 + 16;
-    static constexpr int TMEM_COLS = 4 * NT;               // two accumulator buffers (re, im) x NT
+    static constexpr int TOTAL = BAR_OFF + (2 * RG::RD + 8) * 8 + 16;
+    // two accumulator buffers; at NT = 128 they take all 512 columns, with no room for the hi x lo
+    // terms' own accumulators
+    static constexpr bool SEP = NT <= 64;
 };
 
 template <int NT, int MODE, int SPLIT>
@@ -420,16 +472,18 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
     using LY = PLayout<NT>;
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char* conv = smem;                  // [2][CONV]
-    unsigned char* raw = smem + 2 * RG::CONV;    // [2][RAW]
-    uint64_t* bars = (uint64_t*)(smem + LY::BAR_OFF);
-    uint64_t* raw_full = bars;         // [2] loaders' copies landed (count NLOAD)
-    uint64_t* raw_empty = bars + 2;    // [2] converters done reading (count NCONV)
-    uint64_t* conv_full = bars + 4;    // [2] converted operands written (count NCONV)
-    uint64_t* conv_empty = bars + 6;   // [2] MMAs of the buffer done (tcgen05.commit)
-    uint64_t* acc_full = bars + 8;     // [2] all MMAs of an item's accumulator done (tcgen05.commit)
-    uint64_t* acc_empty = bars + 10;   // [2] epilogue done reading the accumulator (count NEPI)
-    uint32_t* tptr = (uint32_t*)(bars + 12);
-    volatile int* abort = (volatile int*)(bars + 12) + 1;
+    unsigned char* raw = smem + 2 * RG::CONV;    // [RD][RAW]
+    constexpr int RD = RG::RD;
+    constexpr bool SEP = LY::SEP;
+    constexpr int BCOLS = acc_cols<NT, SPLIT, SEP>, TCOLS = 2 * BCOLS;   // one buffer, both
+    uint64_t* raw_full = (uint64_t*)(smem + LY::BAR_OFF);   // [RD] loaders' copies landed (count NLOAD)
+    uint64_t* raw_empty = raw_full + RD;   // [RD] converters done reading (count NCONV)
+    uint64_t* conv_full = raw_empty + RD;  // [2] converted operands written (count NCONV)
+    uint64_t* conv_empty = conv_full + 2;  // [2] MMAs of the buffer done (tcgen05.commit)
+    uint64_t* acc_full = conv_empty + 2;   // [2] all MMAs of an item's accumulator done (tcgen05.commit)
+    uint64_t* acc_empty = acc_full + 2;    // [2] epilogue done reading the accumulator (count NEPI)
+    uint32_t* tptr = (uint32_t*)(acc_empty + 2);
+    volatile int* abort = (volatile int*)tptr + 1;
 
     const int t = threadIdx.x, w = t >> 5, l = t & 31;
     const int mma_warp = (NLOAD + NCONV) / 32;
@@ -437,13 +491,15 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
 
     if (w == mma_warp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(tptr)),
-                     "r"(LY::TMEM_COLS));
+                     "r"(TCOLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (t == 0) {
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < RD; ++b) {
             mbar_init(raw_full + b, NLOAD);
             mbar_init(raw_empty + b, NCONV);
+        }
+        for (int b = 0; b < 2; ++b) {
             mbar_init(conv_full + b, NCONV);
             mbar_init(conv_empty + b, 1);
             mbar_init(acc_full + b, 1);
@@ -475,12 +531,12 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
             Item nxt = cur;
             if (nxt_item < nitems) nxt = decode<NT, MODE>(tasks, jobs, nxt_item, nchunks, KS);
             for (int s = 0; s < cur.nst && ok; ++s, ++gs) {
-                const int slot = (int)(gs & 1);
-                const long long use = gs >> 1;
+                const int slot = (int)(gs % RD);
+                const long long use = gs / RD;
                 Vrows<NT> next_rows;
                 if (s + 1 < cur.nst) next_rows = stage_rows<NT, MODE>(cur, s + 1, t);
                 else if (nxt_item < nitems) next_rows = stage_rows<NT, MODE>(nxt, 0, t);
-                if (gs >= 2) ok = mbar_wait(smem_u32(raw_empty + slot), (uint32_t)((use - 1) & 1), abort, polls);
+                if (gs >= RD) ok = mbar_wait(smem_u32(raw_empty + slot), (uint32_t)((use - 1) & 1), abort, polls);
                 if (!ok) break;
                 load_stage<NT, MODE>(raw + slot * RG::RAW, cur, s, ldc, t, rows);
                 cp_async_arrive(raw_full + slot);
@@ -498,15 +554,15 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
             const int nst = nst_next;   // decoded one item ahead
             if (item + gridDim.x < nitems) nst_next = decode<NT, MODE>(tasks, jobs, item + gridDim.x, nchunks, KS).nst;
             for (int s = 0; s < nst && ok; ++s, ++gs) {
-                const int slot = (int)(gs & 1);
-                const long long use = gs >> 1;
+                const int slot = (int)(gs % RD), cb = (int)(gs & 1);
+                const long long use = gs / RD, cuse = gs >> 1;
                 ok = mbar_wait(smem_u32(raw_full + slot), (uint32_t)(use & 1), abort, polls);
-                if (ok && gs >= 2) ok = mbar_wait(smem_u32(conv_empty + slot), (uint32_t)((use - 1) & 1), abort, polls);
+                if (ok && gs >= 2) ok = mbar_wait(smem_u32(conv_empty + cb), (uint32_t)((cuse - 1) & 1), abort, polls);
                 if (!ok) break;
-                convert_stage<NT, MODE, SPLIT>(raw + slot * RG::RAW, conv + slot * RG::CONV, ct);
+                convert_stage<NT, MODE, SPLIT>(raw + slot * RG::RAW, conv + cb * RG::CONV, ct);
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 mbar_arrive(raw_empty + slot);
-                mbar_arrive(conv_full + slot);
+                mbar_arrive(conv_full + cb);
             }
         }
     } else if (w == mma_warp) {
@@ -522,13 +578,13 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
                 if (nit >= 2) ok = mbar_wait(smem_u32(acc_empty + b), (uint32_t)(((nit >> 1) - 1) & 1), abort, polls);
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t tm_r = tmem + (uint32_t)(b * 2 * NT), tm_i = tm_r + NT;
+                const uint32_t tm = tmem + (uint32_t)(b * BCOLS);
                 for (int s = 0; s < nst && ok; ++s, ++gs) {
                     const int cb = (int)(gs & 1);
                     ok = mbar_wait(smem_u32(conv_full + cb), (uint32_t)((gs >> 1) & 1), abort, polls);
                     if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    mma_stage<NT, SPLIT>(smem_u32(conv + cb * RG::CONV), tm_r, tm_i, s == 0);
+                    mma_item_stage<NT, SPLIT, SEP>(smem_u32(conv + cb * RG::CONV), tm, s == 0);
                     mma_commit(conv_empty + cb);
                 }
                 mma_commit(acc_full + b);   // arrives when every MMA issued so far has completed
@@ -562,11 +618,11 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t lane_off = (uint32_t)(32 * q4) << 16;
-            const uint32_t tm_r = tmem + (uint32_t)(b * 2 * NT) + lane_off, tm_i = tm_r + NT;
+            const uint32_t tm = tmem + (uint32_t)(b * BCOLS) + lane_off;
             for (int c0 = 0; c0 < NT; c0 += 16) {
                 uint32_t vr[16], vi[16];
                 if (it.nst > 0) {
-                    tmem_ld16(tm_r + (uint32_t)c0, tm_i + (uint32_t)c0, vr, vi);
+                    read_acc<NT, SPLIT, SEP>(tm, c0, vr, vi);
                 } else {
 #pragma unroll
                     for (int j = 0; j < 16; ++j) { vr[j] = 0u; vi[j] = 0u; }
@@ -600,7 +656,7 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
     if (!ok && t == 0) atomicExch(flag, 1);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (w == mma_warp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(LY::TMEM_COLS));
+    if (w == mma_warp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(TCOLS));
 }
 
 int sm_count() {
@@ -660,17 +716,20 @@ void launch_mode(const Batch& b, int h, int mode, int ldc, int* flag, cudaStream
 int tc_columns(int ldc) {
     if (ldc % 128 == 0) return 128;
     if (ldc % 64 == 0) return 64;
+    if (ldc % 32 == 0) return 32;
     return 0;
 }
 
 void launch_level_tc(const Batch& b, int h, int mode, int ldc, int* flag, cudaStream_t st) {
-    const bool wide = tc_columns(b.job_cols > 0 ? b.job_cols : ldc) == 128;
+    const int nt = tc_columns(b.job_cols > 0 ? b.job_cols : ldc);
     if (b.split == 1) {
-        if (wide) launch_mode<128, 1>(b, h, mode, ldc, flag, st);
-        else launch_mode<64, 1>(b, h, mode, ldc, flag, st);
+        if (nt == 128) launch_mode<128, 1>(b, h, mode, ldc, flag, st);
+        else if (nt == 64) launch_mode<64, 1>(b, h, mode, ldc, flag, st);
+        else launch_mode<32, 1>(b, h, mode, ldc, flag, st);
     } else {
-        if (wide) launch_mode<128, 3>(b, h, mode, ldc, flag, st);
-        else launch_mode<64, 3>(b, h, mode, ldc, flag, st);
+        if (nt == 128) launch_mode<128, 3>(b, h, mode, ldc, flag, st);
+        else if (nt == 64) launch_mode<64, 3>(b, h, mode, ldc, flag, st);
+        else launch_mode<32, 3>(b, h, mode, ldc, flag, st);
     }
 }
 

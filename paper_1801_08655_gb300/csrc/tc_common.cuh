@@ -148,6 +148,34 @@ __device__ __forceinline__ void mma_stage(uint32_t base, uint32_t tm_r, uint32_t
     }
 }
 
+// The same product with the two halves of the output side by side: one MMA of N = 2 NT computes
+// a real factor part's products with both vector parts, so the factor operand is read from shared
+// memory 6 times per 8 indices instead of 12, and NT = 64 runs at the N = 128 rate.  The vector
+// operand holds [-Xi | Xr | Xi] (3 NT rows) for hi, then for lo; [Yr | Yi] += Ar [Xr | Xi] +
+// Ai [-Xi | Xr], hi x hi terms at tm, the others (SPLIT = 3) at tm + 2 NT.
+template <int NT, int SPLIT>
+__device__ __forceinline__ void mma_stage_wide(uint32_t base, uint32_t tm, bool first_stage) {
+    constexpr int A_MAT = MR * KC * 4, X_MAT = NT * KC * 4;
+    const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(2 * NT >> 3) << 17) | ((uint32_t)(MR >> 4) << 24);
+#pragma unroll
+    for (int ks = 0; ks < KC / 8; ++ks) {
+        const uint32_t ko = ks * 2 * LBO;
+        const uint64_t arh = smem_desc(base + 0 * A_MAT + ko), arl = smem_desc(base + 1 * A_MAT + ko);
+        const uint64_t aih = smem_desc(base + 2 * A_MAT + ko), ail = smem_desc(base + 3 * A_MAT + ko);
+        const uint32_t xb = base + 4 * A_MAT + ko;
+        const uint64_t nrh = smem_desc(xb), rih = smem_desc(xb + X_MAT);   // [-Xi | Xr], [Xr | Xi]
+        const uint32_t first = (first_stage && ks == 0) ? 0u : 1u;
+        mma_tf32(tm, arh, rih, idesc, first);
+        mma_tf32(tm, aih, nrh, idesc, 1u);
+        if (SPLIT == 3) {
+            const uint64_t nrl = smem_desc(xb + 3 * X_MAT), ril = smem_desc(xb + 4 * X_MAT);
+            mma_tf32(tm + 2 * NT, arh, ril, idesc, first);
+            mma_tf32(tm + 2 * NT, arl, rih, idesc, 1u);
+            mma_tf32(tm + 2 * NT, aih, nrl, idesc, 1u);
+            mma_tf32(tm + 2 * NT, ail, nrh, idesc, 1u);
+        }
+    }
+}
 
 }  // namespace tcc
 }  // namespace hz

@@ -13,6 +13,18 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
+def solve_and_compare(s, shape, m, omega, npml, C, cols, rng):
+    nz, ny, nx = shape
+    A = D.assemble(m, omega, *[D.global_profiles(n, npml, C, omega) for n in (nx, ny, nz)]).tocsc()
+    lu = spla.splu(A)
+    for R in cols:
+        g = rng.standard_normal((R,) + shape) + 1j * rng.standard_normal((R,) + shape)
+        ref = lu.solve(np.ascontiguousarray(g.reshape(R, -1).T)).T.reshape(g.shape)
+        w = s.layer_solve(0, torch.from_numpy(g).cuda()).cpu().numpy()
+        err = np.linalg.norm(w - ref) / np.linalg.norm(ref)
+        assert err < 2e-4, (R, err)
+
+
 @pytest.mark.parametrize("shape,leaf,tc_min,cols", [
     ((4, 5, 7), 1000, 128, (1, 3)),        # a single node of 140 unknowns: no update rows
     ((3, 4, 9), 8, 1, (2,)),               # nodes of a few cells
@@ -32,12 +44,25 @@ def test_layer_solve_on_m21(shape, leaf, tc_min, cols, precision, monkeypatch):
     m, omega, npml, C = 1.0 / (c * c), W.omega_for_ppw(1.5, 9.0), 1, W.pml_constant(2.5)
     s = hz.Solver(m, omega, npml, C, 1, precision=precision)
     s.factor()
-    prof = [D.global_profiles(n, npml, C, omega) for n in (nx, ny, nz)]
-    A = D.assemble(m, omega, *prof).tocsc()
-    for R in cols:
-        g = rng.standard_normal((R,) + shape) + 1j * rng.standard_normal((R,) + shape)
-        ref = spla.spsolve(A, g.reshape(R, -1).T).reshape(nz * ny * nx, R).T.reshape(g.shape)
-        w = s.layer_solve(0, torch.from_numpy(g).cuda()).cpu().numpy()
-        err = np.linalg.norm(w - ref) / np.linalg.norm(ref)
-        assert err < 2e-4, (R, err)
+    solve_and_compare(s, shape, m, omega, npml, C, cols, rng)
+    s.close()
+
+
+@pytest.mark.parametrize("shape", [(21, 24, 23), (9, 33, 10)])
+@pytest.mark.parametrize("cfg", [0, 1])
+def test_narrow_column_blocks_on_the_tensor_cores(shape, cfg, monkeypatch):
+    """17 to 128 columns (tiles of 32, 64 and 128) forced onto the tensor-core kernels."""
+    from paper_1801_08655_gb300 import build, hz
+    build.build()
+    for k, v in (("HZ_SUBST_TC", 1), ("HZ_TC_MIN_TILES", 2), ("HZ_AUTOTUNE", 0), ("HZ_TC_CFG", cfg)):
+        monkeypatch.setenv(k, str(v))
+    rng = np.random.default_rng(sum(shape) + cfg)
+    c = 1.5 + rng.random(shape)
+    m, omega, npml, C = 1.0 / (c * c), W.omega_for_ppw(1.5, 9.0), 1, W.pml_constant(2.5)
+    s = hz.Solver(m, omega, npml, C, 1, precision="mixed")
+    s.factor()
+    s.profile_begin(detail=True)
+    solve_and_compare(s, shape, m, omega, npml, C, (17, 32, 33, 128), rng)
+    s.profile_end()
+    assert s.profile_kernel(1)["launches"] > 0
     s.close()
