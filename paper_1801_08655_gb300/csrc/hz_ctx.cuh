@@ -34,6 +34,15 @@ struct ZeroDev { void* p; long long bytes; };
 // Clears n vectors, the longest of max_bytes, in one launch.
 void launch_zero(const ZeroDev* d, int n, long long max_bytes, cudaStream_t st);
 
+// Task lists of the one-launch substitution (subst_stream.cu): tasks ordered by warp and phase,
+// off[warp * nph + phase] the first one of each.
+struct StreamPlan {
+    void* d_tasks = nullptr;
+    int* d_off = nullptr;
+    int nph = 0, grid = 0;
+};
+struct StreamProduct { int mode, level, job, node; };
+
 // A set of layers solved together (one job per layer) with its per-level task lists.
 struct Batch {
     std::vector<int> layers;
@@ -51,6 +60,8 @@ struct Batch {
                                                 // layer's columns into jobs (0: one job per layer, ldc wide)
     long long wait_polls = 1LL << 26;           // poll limit of the tensor-core kernels' pipeline waits
     std::vector<long long> pair_off[4], pair_cnt[4];  // tensor-core tasks: two output tiles each
+    bool stream = false;                        // runs as one cooperative launch (plan below)
+    StreamPlan plan;
     Task* d_tasks = nullptr;
     void* d_jobs = nullptr;                     // JobDev<C>[njobs]
     std::vector<std::pair<void*, void*>> vec_ptrs;  // (acc, x) of each layer
@@ -221,6 +232,7 @@ struct Ctx {
     std::vector<std::string> tune_log;
     int tc_mode = 2;        // tensor-core substitution (complex64, >= 64 columns): 0 never, 1 always,
                             // 2 when the autotuner measures it faster for the batch signature
+    bool one_launch = true; // complex64 substitutions of at most 16 columns as one launch (HZ_ONE_LAUNCH)
     int tc_ks = 4;          // split-K (factor tiles per block) of small tensor-core batches
     int tc_min_tiles = 8;   // output tiles a node product needs to run on the tensor cores
     int tc_cfg = 0;         // untuned tensor-core kernel: 0 one block per work item, 1 persistent (HZ_TC_CFG)

@@ -10,6 +10,13 @@ int chunk_cols(bool is_double, int ncols);
 int tc_columns(int ldc);   // tensor-core column tile for this leading dimension (0: not usable)
 void launch_level_tc(const Batch& b, int h, int mode, int ldc, int* flag, cudaStream_t st);
 int padded_ldc(bool is_double, int ncols);
+// one-launch substitution of complex64 blocks (subst_stream.cu): usable for this leading dimension;
+// task lists of a batch's active products; the launch (sync: two counters, zero between launches)
+bool stream_usable(int ldc);
+void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vector<StreamProduct>& prods, int H,
+                  StreamPlan& plan);
+void launch_stream(const StreamPlan& p, const void* jobs, int ldc, unsigned* sync, int* flag, long long polls,
+                   cudaStream_t st);
 
 // Sparsity of a batch: which planes of each layer carry the sources (forward code, bits 0-1) and
 // the read-outs (backward code, bits 2-3).  SP_ALL: anywhere (no product skipped); SP_BOTH: the
@@ -37,7 +44,8 @@ inline int block_code(int sparse, int q) { return (sparse & SP_BLOCKS) ? (sparse
 template <class C> Batch& get_batch(Ctx& ctx, const std::vector<int>& layers, int ncols, int split = 3, int sparse = 0);
 // Build (or fetch) a batch with an explicit split-K depth and column chunk.
 template <class C> Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS, int CC, bool tc,
-                                       int KS_tc, int min_t, int split = 3, int tc_cfg = 0, int sparse = 0);
+                                       int KS_tc, int min_t, int split = 3, int tc_cfg = 0, int sparse = 0,
+                                       bool stream = false);
 // Autotune the substitution of this batch signature (times candidate split-K depths and column
 // chunks on zeroed slot vectors); a no-op once the signature is tuned or when tuning is off.
 template <class C> void ensure_tuned(Ctx& ctx, const std::vector<int>& layers, int ncols, int split = 3,

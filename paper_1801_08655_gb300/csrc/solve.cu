@@ -401,6 +401,12 @@ struct LaunchTimer {
 
 template <class C, int CC>
 void run_batch(const Batch& b, int ldc, int ncols, bool tc, int* flag, cudaStream_t st, std::vector<ProfRec>* pl) {
+    if (b.stream) {
+        LaunchTimer lt(pl, st, 0, b.alg_bytes, b.flops_per_col * ncols, FA, 0, b.plan.nph);
+        launch_stream(b.plan, b.d_jobs, ldc, (unsigned*)(flag + 1), flag, b.wait_polls, st);
+        lt.done();
+        return;
+    }
     auto level = [&](int h, int mode) {
         if (b.cnt[mode][h] > 0) {
             LaunchTimer lt(pl, st, 0, b.lvl_bytes[0][mode][h], b.lvl_flops[0][mode][h] * ncols, mode, h, b.cnt[mode][h]);
@@ -446,8 +452,9 @@ void launch_zero(const ZeroDev* d, int n, long long max_bytes, cudaStream_t st) 
 }
 
 int chunk_cols(bool is_double, int ncols) {
+    // complex64 columns come in pairs: 16-byte vector accesses
     const int cmax = is_double ? 32 : 64;
-    int c = 1;
+    int c = is_double ? 1 : 2;
     while (c < ncols && c < cmax) c *= 2;
     return c;
 }
@@ -508,6 +515,13 @@ static bool tc_usable(const Ctx& ctx, int ldc) {
     return nt > 32 || (nt == 32 && ctx.prec == HZ_PREC_MIXED);
 }
 
+// Complex64 blocks of at most 16 columns run as one launch (subst_stream.cu): faster than the launches
+// per phase at every width, tree and layer set measured (24^3 to 64^3, one layer: 1.5-1.9x, all
+// layers: 1.3-1.7x), so nothing is timed for them.
+static bool use_one_launch(const Ctx& ctx, int ldc, int sparse) {
+    return ctx.one_launch && stream_usable(ldc) && block_count(sparse) == 1;
+}
+
 static std::string tune_key(const Ctx& ctx, const std::vector<int>& layers, int ldc, int split, int sparse) {
     std::vector<int> shapes;
     for (int l : layers) shapes.push_back(ctx.layers[l].shape);
@@ -528,6 +542,8 @@ Batch& get_batch(Ctx& ctx, const std::vector<int>& layers, int ncols, int split,
         return get_batch_cfg<C>(ctx, layers, ncols, ch.KS, ch.CC, tc_ok && ch.tc, ch.KS_tc, ch.min_t, split, ch.tc_cfg,
                                 sparse);
     }
+    if (!dbl && use_one_launch(ctx, ldc, sparse))
+        return get_batch_cfg<C>(ctx, layers, ncols, 0, 0, false, 1 << 30, 0, split, 0, sparse, true);
     // default: split the reductions when the batch alone cannot fill the GPU
     const int nchunks = ldc / chunk_cols(dbl, ncols);
     const int KS = ((long long)layers.size() * nchunks >= 64) ? (1 << 30) : 8;
@@ -544,6 +560,7 @@ void ensure_tuned(Ctx& ctx, const std::vector<int>& layers, int ncols, int split
     const bool tc_ok = !dbl && tc_usable(ctx, ldc);
     const std::string key = tune_key(ctx, layers, ldc, split, sparse);
     if (!ctx.autotune || ctx.tuned.count(key)) return;
+    if (!dbl && use_one_launch(ctx, ldc, sparse)) return;   // get_batch takes it without timing
     const int cc0 = chunk_cols(dbl, ncols);
     std::vector<Ctx::TuneChoice> cands;
     const bool try_tc = tc_ok && ctx.tc_mode >= 1;
@@ -602,13 +619,13 @@ void ensure_tuned(Ctx& ctx, const std::vector<int>& layers, int ncols, int split
 
 template <class C>
 Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS, int CC, bool tc, int KS_tc,
-                     int min_t, int split, int tc_cfg, int sparse) {
+                     int min_t, int split, int tc_cfg, int sparse, bool stream) {
     const bool dbl = sizeof(C) == 16;
     const int ldc = padded_ldc(dbl, ncols);
     std::string key = "KS" + std::to_string(KS) + "C" + std::to_string(CC) + "n" + std::to_string(ldc) +
                       (tc ? "tc" + std::to_string(KS_tc) + "m" + std::to_string(min_t) + "s" + std::to_string(split) +
                                 "c" + std::to_string(tc_cfg)
-                          : "") + "p" + std::to_string(sparse) + ":";
+                          : stream ? "st" : "") + "p" + std::to_string(sparse) + ":";
     for (int l : layers) key += std::to_string(l) + ",";
     auto it = ctx.batches.find(key);
     if (it != ctx.batches.end()) return it->second;
@@ -623,6 +640,8 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
     b.tc_cfg = tc_cfg;
     b.sparse = sparse;
     b.wait_polls = ctx.tc_wait_polls;
+    b.stream = stream;
+    std::vector<StreamProduct> prods;
     // per-block sparsity: job j * nblk + q is block q (columns [q * job_cols, (q + 1) * job_cols))
     // of layer j; the caller has checked that the blocks tile the columns in whole chunks
     const int nblk = block_count(sparse);
@@ -694,7 +713,9 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
                         if (!on) continue;
                         ++nact;
                         const int jq = j * nblk + q;
-                        if (on_tc) {
+                        if (stream) {
+                            prods.push_back({mode, h, jq, nid});
+                        } else if (on_tc) {
                             for (int t = 0; t < out_t; t += 4) {
                                 if (mode == 0) add_tasks(quads[0][hl], jq, nid, t, 0, std::min(t + 4, nd.own_t), b.KS_tc);
                                 if (mode == 1) add_tasks(quads[1][hl], jq, nid, t, 0, nd.own_t, b.KS_tc);
@@ -788,6 +809,7 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
                 b.alg_bytes += b.lvl_bytes[k][mode][h];
                 b.flops_per_col += b.lvl_flops[k][mode][h];
             }
+    if (stream) build_stream(ctx, layers, prods, H, b.plan);
     for (int w = 0; w < 2; ++w) {
         std::vector<ZeroDev> zd;
         for (size_t j = 0; j < b.vec_ptrs.size(); ++j) {
@@ -810,6 +832,8 @@ void free_batches(Ctx& ctx) {
     for (auto& kv : ctx.batches) {
         cudaFree(kv.second.d_tasks);
         cudaFree(kv.second.d_jobs);
+        cudaFree(kv.second.plan.d_tasks);
+        cudaFree(kv.second.plan.d_off);
         cudaFree(kv.second.d_zero[0]);
         cudaFree(kv.second.d_zero[1]);
     }
@@ -820,8 +844,8 @@ template void substitute<float2>(Ctx&, const Batch&, int, cudaStream_t);
 template void substitute<double2>(Ctx&, const Batch&, int, cudaStream_t);
 template Batch& get_batch<float2>(Ctx&, const std::vector<int>&, int, int, int);
 template Batch& get_batch<double2>(Ctx&, const std::vector<int>&, int, int, int);
-template Batch& get_batch_cfg<float2>(Ctx&, const std::vector<int>&, int, int, int, bool, int, int, int, int, int);
-template Batch& get_batch_cfg<double2>(Ctx&, const std::vector<int>&, int, int, int, bool, int, int, int, int, int);
+template Batch& get_batch_cfg<float2>(Ctx&, const std::vector<int>&, int, int, int, bool, int, int, int, int, int, bool);
+template Batch& get_batch_cfg<double2>(Ctx&, const std::vector<int>&, int, int, int, bool, int, int, int, int, int, bool);
 template void ensure_tuned<float2>(Ctx&, const std::vector<int>&, int, int, int);
 template void ensure_tuned<double2>(Ctx&, const std::vector<int>&, int, int, int);
 

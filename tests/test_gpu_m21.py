@@ -66,3 +66,53 @@ def test_narrow_column_blocks_on_the_tensor_cores(shape, cfg, monkeypatch):
     s.profile_end()
     assert s.profile_kernel(1)["launches"] > 0
     s.close()
+
+
+@pytest.mark.parametrize("shape,leaf", [((4, 5, 7), 1000), ((3, 4, 9), 8), ((9, 33, 10), 64), ((21, 24, 23), 256),
+                                        ((12, 40, 44), 2000)])
+def test_one_launch_substitution(shape, leaf, monkeypatch):
+    """1 to 16 columns forced onto the one-launch kernel: one-node and one-tile trees, ragged tiles,
+    split and whole reductions (the last box has nodes of over 8 half tiles)."""
+    from paper_1801_08655_gb300 import build, hz
+    build.build()
+    monkeypatch.setenv("HZ_ONE_LAUNCH", "1")
+    monkeypatch.setenv("HZ_LEAF", str(leaf))
+    rng = np.random.default_rng(sum(shape))
+    c = 1.5 + rng.random(shape)
+    m, omega, npml, C = 1.0 / (c * c), W.omega_for_ppw(1.5, 9.0), 1, W.pml_constant(2.5)
+    s = hz.Solver(m, omega, npml, C, 1, precision="mixed")
+    s.factor()
+    solve_and_compare(s, shape, m, omega, npml, C, (1, 2, 3, 8, 13, 16, 1), rng)
+    s.close()
+
+
+def test_one_launch_sparse_products_and_timeout(monkeypatch):
+    """The trace operators' batches (skipped subtrees, several layers) agree with the per-phase launches;
+    a wait that gives up is a status and leaves the counters usable for the next handle."""
+    from paper_1801_08655_gb300 import build, hz
+    build.build()
+    p = W.small_problem(26, 4, 4, seed=5, R=3)
+    out = {}
+    for mode in ("0", "1"):
+        monkeypatch.setenv("HZ_ONE_LAUNCH", mode)
+        s = hz.Solver(p.m, p.omega, p.npml, p.C, p.n_layers, precision="mixed")
+        s.factor()
+        x = torch.randn(s.trace_shape(3), dtype=torch.complex128, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+        f = torch.from_numpy(p.rhs()).cuda()
+        out[mode] = [s.apply_mpol(x), s.apply_precond(x), s.polarized_rhs(f), s.solve(f)[0]]
+        s.close()
+    for a, b in zip(out["0"], out["1"]):
+        assert float((a - b).norm() / b.norm()) < 1e-5   # FP32 rounding, other summation orders
+    monkeypatch.setenv("HZ_FACTOR_TC_MIN", "0")   # no bounded waits in the factorization
+    ok = hz.Solver(p.m, p.omega, p.npml, p.C, p.n_layers, precision="mixed")
+    ok.factor()
+    monkeypatch.setenv("HZ_TC_WAIT_POLLS", "1")
+    s = hz.Solver(p.m, p.omega, p.npml, p.C, p.n_layers, precision="mixed")
+    s.factor()
+    with pytest.raises(hz.HzError) as e:
+        s.solve(f)
+    assert e.value.status == hz.HZ_ERR_TIMEOUT
+    u = ok.solve(f)[0]
+    assert float((u - out["1"][3]).norm() / u.norm()) < 1e-5
+    s.close()
+    ok.close()
