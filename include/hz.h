@@ -74,7 +74,9 @@ typedef struct {
                             pass solves to 0.1 refine_tol / (its starting volume residual), capped at 0.1 */
     int32_t restart;     /* Krylov dimension before restart (default 12) */
     int32_t max_iter;    /* total GMRES iterations cap (default 100) */
-    double refine_tol;   /* mixed mode: stop refining when ||S f - A u|| <= refine_tol ||S f|| (default 1e-9) */
+    double refine_tol;   /* mixed mode: refine until ||S f - A u|| <= refine_tol ||S f|| (default 1e-9).  A pass
+                            is added while the residual is above half of it, above a tenth of it where no
+                            correction has been made yet, so that a borderline pass is not the last one */
     int32_t max_refine;  /* mixed mode: maximum defect-correction passes (default 3) */
     int32_t krylov;      /* Krylov solver on the trace system: 0 GMRES(restart) (default), 1 Bi-CGSTAB
                             (two products P M_pol per iteration, six trace vectors per column instead
