@@ -65,8 +65,9 @@ struct Batch {
     Task* d_tasks = nullptr;
     void* d_jobs = nullptr;                     // JobDev<C>[njobs]
     std::vector<std::pair<void*, void*>> vec_ptrs;  // (acc, x) of each layer
-    ZeroDev* d_zero[2] = {nullptr, nullptr};        // acc / x vectors of every layer, for launch_zero
-    long long zero_max = 0;                         // bytes of the longest of them
+    ZeroDev* d_zero[2] = {nullptr, nullptr};        // rows of acc / x to clear, for launch_zero
+    int zero_n[2] = {0, 0};
+    long long zero_max = 0;                         // bytes of the longest entry
     std::vector<long long> vec_rows;
     double alg_bytes = 0;       // factor bytes one forward+backward substitution streams (all jobs)
     double flops_per_col = 0;   // real flops per right-hand-side column (all jobs)

@@ -155,7 +155,8 @@ template <class C> struct JobDev {
     C* x;     // solution
 };
 
-struct Task { int job, node, tile, pad_; };
+// One output tile (four on the tensor cores) of a node product over reduction tiles [k0, k0 + klen).
+struct Task { int job, node, tile; unsigned short k0, klen; };
 
 // ------------------------------------------------------------------------------------------
 // error handling

@@ -50,23 +50,50 @@ template <class C> struct Inject {
 // Trace vectors keep cells contiguous per right-hand side; the slot vectors keep right-hand sides
 // contiguous per row.  The three kernels below move a tile of 32 cells x 32 right-hand sides
 // through shared memory so that both sides are read and written along their contiguous index
-// (tile[a][b] with a pitch of 33 16-byte elements: conflict-free along either index).
+// (tile[a][b] with a pitch of 33 16-byte elements: conflict-free along either index).  What depends on the
+// cell alone (row, FP64 weight) is formed once per cell, by one warp beside the loads: formed per
+// element it was most of the FP64 work that bound them (64^3, 16 columns: volume source 172 us,
+// injection 28 us; a 64^3 solve with 16 columns 43.5 -> 40.9 ms with this and the sweeps' batched
+// clearing, 128^3 with 32 columns 932 -> 894 ms).  With fewer right-hand sides than lanes, a warp takes several cells at once.
 constexpr int IO_T = 32;
+
+// lanes along the right-hand sides of a tile: the smallest power of two that holds them
+__device__ __forceinline__ int io_lanes_shift(int nr) { return nr >= 32 ? 5 : 32 - __clz(max(nr, 1) - 1); }
+
+// a * b, as two products where a is real (the physical box: no stretch)
+__device__ __forceinline__ double2 cmul_real_aware(double2 a, double2 b) {
+    return a.y == 0.0 ? make_double2(a.x * b.x, a.x * b.y) : cmul(a, b);
+}
 
 template <class C>
 __global__ void __launch_bounds__(256) k_inject(const Inject<C>* inj, const double2* sx, const double2* sy,
                                                 double inv_h2, int nx, int ny, int R) {
     __shared__ double2 tm[IO_T][IO_T + 1], tp[IO_T][IO_T + 1];   // [r][cell]
+    __shared__ double2 cs[IO_T];
+    __shared__ int pm[IO_T], pp[IO_T];
     const Inject<C> q = inj[blockIdx.z];
     const int P = nx * ny;
     const int cell0 = blockIdx.x * IO_T, r0 = blockIdx.y * IO_T;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int nr = min(IO_T, R - r0);
+    if (w == 7) {
+        const int cell = cell0 + lane;
+        if (cell < P) {
+            // c = A[(Q,y,x),(P,y,x)]: the z-coupling across the physical half plane between the pair's
+            // planes (zl_m and zl_p are the two of them), times b at that half plane
+            double2 c = cscale(cmul(sx[cell % nx], sy[cell / nx]), inv_h2);
+            if (q.b) c = cscale(c, 0.5 * (q.b[(long long)q.zl_m * P + cell] + q.b[(long long)q.zl_p * P + cell]));
+            cs[lane] = c;
+            pm[lane] = q.pos[q.zl_m * P + cell];
+            pp[lane] = q.pos[q.zl_p * P + cell];
+        }
+    }
     // trace planes, read along cells
-    for (int rr = w; rr < IO_T; rr += 8) {
-        const int r = r0 + rr, cell = cell0 + lane;
+    for (int rr = w; rr < nr; rr += 8) {
+        const int cell = cell0 + lane;
         double2 vm = make_double2(0.0, 0.0), vp = vm;
-        if (r < R && cell < P) {
-            const double2* src = q.src + (long long)r * q.rstride;
+        if (cell < P) {
+            const double2* src = q.src + (long long)(r0 + rr) * q.rstride;
             vm = src[q.off_m + cell];
             vp = src[q.off_p + cell];
         }
@@ -75,18 +102,13 @@ __global__ void __launch_bounds__(256) k_inject(const Inject<C>* inj, const doub
     }
     __syncthreads();
     // slot rows, written along the right-hand sides
-    const int r = r0 + lane;
-    for (int cc = w; cc < IO_T; cc += 8) {
-        const int cell = cell0 + cc;
-        if (cell >= P) break;
-        if (r >= R) continue;
-        const int x = cell % nx, y = cell / nx;
-        // c = A[(Q,y,x),(P,y,x)]: the z-coupling across the physical half plane between the pair's
-        // planes (zl_m and zl_p are the two of them), times b at that half plane
-        double2 c = cscale(cmul(sx[x], sy[y]), inv_h2);
-        if (q.b) c = cscale(c, 0.5 * (q.b[(long long)q.zl_m * P + cell] + q.b[(long long)q.zl_p * P + cell]));
-        atomic_addc(q.acc + (long long)q.pos[q.zl_m * P + cell] * q.ldc + q.col0 + r, cneg(cmul(c, tm[lane][cc])));
-        atomic_addc(q.acc + (long long)q.pos[q.zl_p * P + cell] * q.ldc + q.col0 + r, cmul(c, tp[lane][cc]));
+    const int sh = io_lanes_shift(nr), rr = lane & ((1 << sh) - 1);
+    for (int cc = (w << (5 - sh)) + (lane >> sh); cc < IO_T; cc += 8 << (5 - sh)) {
+        if (cell0 + cc >= P || rr >= nr) continue;
+        const double2 c = cs[cc];
+        const int col = q.col0 + r0 + rr;
+        atomic_addc(q.acc + (long long)pm[cc] * q.ldc + col, cneg(cmul_real_aware(c, tm[rr][cc])));
+        atomic_addc(q.acc + (long long)pp[cc] * q.ldc + col, cmul_real_aware(c, tp[rr][cc]));
     }
 }
 
@@ -106,24 +128,24 @@ __global__ void __launch_bounds__(256) k_extract(const Extract<C>* ex, int P, in
     const Extract<C> q = ex[blockIdx.z];
     const int cell0 = blockIdx.x * IO_T, r0 = blockIdx.y * IO_T;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int nr = min(IO_T, R - r0);
     // slot rows, read along the right-hand sides (the column blocks summed)
-    for (int cc = w; cc < IO_T; cc += 8) {
-        const int cell = cell0 + cc, r = r0 + lane;
+    const int sh = io_lanes_shift(nr), rl = lane & ((1 << sh) - 1);
+    for (int cc = (w << (5 - sh)) + (lane >> sh); cc < IO_T; cc += 8 << (5 - sh)) {
+        const int cell = cell0 + cc;
         double2 v = make_double2(0.0, 0.0);
-        if (cell < P && r < R) {
-            const C* xr = q.x + (long long)q.pos[q.zl * P + cell] * q.ldc + r;
+        if (cell < P && rl < nr) {
+            const C* xr = q.x + (long long)q.pos[q.zl * P + cell] * q.ldc + r0 + rl;
             for (int b = 0; b < q.nblk; ++b) v = cadd(v, to_d(xr[q.cols[b]]));
         }
-        t[cc][lane] = v;
+        t[cc][rl] = v;
     }
     __syncthreads();
     // trace plane, updated along cells
     const int cell = cell0 + lane;
-    for (int rr = w; rr < IO_T; rr += 8) {
-        const int r = r0 + rr;
-        if (r >= R) break;
+    for (int rr = w; rr < nr; rr += 8) {
         if (cell >= P) continue;
-        double2* d = q.dst + (long long)r * q.rstride + cell;
+        double2* d = q.dst + (long long)(r0 + rr) * q.rstride + cell;
         *d = cadd(*d, cscale(t[lane][rr], q.sign));
     }
 }
@@ -142,6 +164,8 @@ __global__ void __launch_bounds__(256) k_volume_source(const VolIO<C>* io, const
                                                        int nx, int ny, const double2* sx, const double2* sy,
                                                        const double2* sz, int scale) {
     __shared__ double2 t[IO_T][IO_T + 1];   // [r][cell]
+    __shared__ double2 Ss[IO_T];
+    __shared__ int ps[IO_T];
     if (gslot) g = *gslot;   // recorded plans read the caller's volume through the handle's slot
     const VolIO<C> q = io[blockIdx.z];
     const int P = nx * ny;
@@ -149,19 +173,21 @@ __global__ void __launch_bounds__(256) k_volume_source(const VolIO<C>* io, const
     if (z > q.hi) return;   // uniform over the block
     const int cell0 = blockIdx.x * IO_T, r0 = ((int)blockIdx.y % nrt) * IO_T;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int rr = w; rr < IO_T; rr += 8) {   // volume, read along cells
-        const int r = r0 + rr, cell = cell0 + lane;
-        t[rr][lane] = (r < R && cell < P) ? g[(long long)r * N3 + (long long)z * P + cell] : make_double2(0.0, 0.0);
+    const int nr = min(IO_T, R - r0);
+    if (w == 7 && cell0 + lane < P) {
+        const int cell = cell0 + lane;
+        Ss[lane] = scale ? cmul(cmul(sx[cell % nx], sy[cell / nx]), sz[z]) : make_double2(1.0, 0.0);
+        ps[lane] = q.pos[(z - q.zlo) * P + cell];
+    }
+    for (int rr = w; rr < nr; rr += 8) {   // volume, read along cells
+        const int cell = cell0 + lane;
+        t[rr][lane] = cell < P ? g[(long long)(r0 + rr) * N3 + (long long)z * P + cell] : make_double2(0.0, 0.0);
     }
     __syncthreads();
-    const int r = r0 + lane;
-    for (int cc = w; cc < IO_T; cc += 8) {   // slot rows, written along the right-hand sides
-        const int cell = cell0 + cc;
-        if (cell >= P) break;
-        if (r >= R) continue;
-        double2 S = make_double2(1.0, 0.0);
-        if (scale) S = cmul(cmul(sx[cell % nx], sy[cell / nx]), sz[z]);
-        q.vec[(long long)q.pos[(z - q.zlo) * P + cell] * q.ldc + q.col0 + r] = from_d<C>(cmul(S, t[lane][cc]));
+    const int sh = io_lanes_shift(nr), rr = lane & ((1 << sh) - 1);
+    for (int cc = (w << (5 - sh)) + (lane >> sh); cc < IO_T; cc += 8 << (5 - sh)) {   // slot rows, along the right-hand sides
+        if (cell0 + cc >= P || rr >= nr) continue;
+        q.vec[(long long)ps[cc] * q.ldc + q.col0 + r0 + rr] = from_d<C>(cmul_real_aware(Ss[cc], t[rr][cc]));
     }
 }
 
@@ -441,12 +467,23 @@ __global__ void k_store_blocks(C* base, const long long* off, const double2* T, 
 // ------------------------------------------------------------------------------------------
 // FP64 volume residual r = g - A u, g = S f (scale) or f, with per-column norms
 // ------------------------------------------------------------------------------------------
+// r -= c v, and the same for a real c
+__device__ __forceinline__ void cfms(double2& r, double2 c, double2 v) {
+    r.x = fma(-c.x, v.x, r.x); r.x = fma(c.y, v.y, r.x);
+    r.y = fma(-c.x, v.y, r.y); r.y = fma(-c.y, v.x, r.y);
+}
+__device__ __forceinline__ void rfms(double2& r, double2 c, double2 v) {
+    r.x = fma(-c.x, v.x, r.x);
+    r.y = fma(-c.x, v.y, r.y);
+}
+
 template <int RB>
 __global__ void __launch_bounds__(256) k_residual(const double2* f, const double2* u, double2* rout, double* norms,
                                                   int scale, int R, int nx, int ny, int nz, const double2* sxn,
                                                   const double2* isxh, const double2* syn, const double2* isyh,
                                                   const double2* szn, const double2* iszh, const double* m,
                                                   const double* b, double omega2, double inv_h2) {
+    // (128^3, 16 columns: 4.23 ms with separate products and sums, 3.24 ms as fused chains)
     // one cell and RB columns per thread: the cell's stencil coefficients (FP64, as in the
     // assembly) are formed once and applied to RB columns, so that the FP64 pipe (the bound of
     // this kernel on a GPU whose FP64 rate is a small fraction of its FP32 rate) spends its
@@ -485,24 +522,31 @@ __global__ void __launch_bounds__(256) k_residual(const double2* f, const double
         if (y == ny - 1) c4 = zero;
         if (z == 0) c5 = zero;
         if (z == nz - 1) c6 = zero;
+        // no stretch here or at the neighbours: every coefficient is real (whole warps take one side)
+        const bool real = __all_sync(__activemask(), sxyz.y == 0.0 && dg.y == 0.0 && c1.y == 0.0 && c2.y == 0.0 &&
+                                                         c3.y == 0.0 && c4.y == 0.0 && c5.y == 0.0 && c6.y == 0.0);
 #pragma unroll
         for (int j = 0; j < RB; ++j) {
             const int r = r0 + j;
             if (r >= R) break;
             const double2* ur = u + (long long)r * N3;
-            double2 au = cmul(dg, ur[i]);
-            au = cadd(au, cmul(c1, ur[ix0]));
-            au = cadd(au, cmul(c2, ur[ix1]));
-            au = cadd(au, cmul(c3, ur[iy0]));
-            au = cadd(au, cmul(c4, ur[iy1]));
-            au = cadd(au, cmul(c5, ur[iz0]));
-            au = cadd(au, cmul(c6, ur[iz1]));
             double2 g = f[(long long)r * N3 + i];
-            if (scale) g = cmul(sxyz, g);
-            const double2 res = csub(g, au);
+            if (scale) g = real ? cscale(g, sxyz.x) : cmul(sxyz, g);
+            double2 res = g;   // g - A u, one fused chain per part
+            if (real) {
+                rfms(res, dg, ur[i]);
+                rfms(res, c1, ur[ix0]); rfms(res, c2, ur[ix1]);
+                rfms(res, c3, ur[iy0]); rfms(res, c4, ur[iy1]);
+                rfms(res, c5, ur[iz0]); rfms(res, c6, ur[iz1]);
+            } else {
+                cfms(res, dg, ur[i]);
+                cfms(res, c1, ur[ix0]); cfms(res, c2, ur[ix1]);
+                cfms(res, c3, ur[iy0]); cfms(res, c4, ur[iy1]);
+                cfms(res, c5, ur[iz0]); cfms(res, c6, ur[iz1]);
+            }
             if (rout) rout[(long long)r * N3 + i] = res;
-            rr[j] = res.x * res.x + res.y * res.y;
-            gg[j] = g.x * g.x + g.y * g.y;
+            rr[j] = fma(res.x, res.x, res.y * res.y);
+            gg[j] = fma(g.x, g.x, g.y * g.y);
         }
     }
     // block reductions of the RB column pairs, one atomic pair per column and block
@@ -752,6 +796,7 @@ void rec_zero_slots(Ctx& ctx, Rec& rec, const std::vector<int>& layers, int ldc)
         zd.push_back({ctx.slot_acc[l], ctx.shapes[ctx.layers[l].shape].N * ldc * (long long)sizeof(C)});
         most = std::max(most, zd.back().bytes);
     }
+    if (zd.empty()) return;
     const ZeroDev* d = rec.up(zd);
     const int n = (int)zd.size();
     rec.add([=](cudaStream_t st) { launch_zero(d, n, most, st); });
@@ -1077,9 +1122,8 @@ template <class C>
 void rec_apply_precond_blocks(Ctx& ctx, Rec& rec, const double2* x, int R, double2* y, double2* tmp) {
     const int K = ctx.K, L = ctx.L;
     const long long ntr = ctx.ntr;
-    rec_pairs_axpy(ctx, rec, pair_ptr(y, ctx, 0, 0), ntr, pair_ptr(x, ctx, 0, 0), ntr, -1.0, nullptr, 0, 0.0, 0, 1, R);
+    rec_pairs_axpy(ctx, rec, pair_ptr(y, ctx, 0, 0), ntr, pair_ptr(x, ctx, 0, 0), ntr, -1.0, nullptr, 0, 0.0, 0, K, R);
     for (int j = 1; j < K; ++j) {
-        rec_pairs_axpy(ctx, rec, pair_ptr(y, ctx, 0, j), ntr, pair_ptr(x, ctx, 0, j), ntr, -1.0, nullptr, 0, 0.0, 0, 1, R);
         TBJob<C> jb = tb_job<C>(pair_ptr(y, ctx, 0, j), 1.0);
         tb_term(jb, trace_block<C>(ctx, j, 1, 0), pair_ptr(y, ctx, 0, j - 1));
         rec_trace_blocks<C>(ctx, rec, {jb}, R);
@@ -1097,9 +1141,8 @@ void rec_apply_precond_blocks(Ctx& ctx, Rec& rec, const double2* x, int R, doubl
         }
         rec_trace_blocks<C>(ctx, rec, jobs, R);
     }
-    rec_pairs_axpy(ctx, rec, pair_ptr(y, ctx, 1, K - 1), ntr, pair_ptr(s, ctx, 1, K - 1), ntr, -1.0, nullptr, 0, 0.0, 0, 1, R);
+    rec_pairs_axpy(ctx, rec, pair_ptr(y, ctx, 1, 0), ntr, pair_ptr(s, ctx, 1, 0), ntr, -1.0, nullptr, 0, 0.0, 0, K, R);
     for (int j = K - 2; j >= 0; --j) {
-        rec_pairs_axpy(ctx, rec, pair_ptr(y, ctx, 1, j), ntr, pair_ptr(s, ctx, 1, j), ntr, -1.0, nullptr, 0, 0.0, 0, 1, R);
         TBJob<C> jb = tb_job<C>(pair_ptr(y, ctx, 1, j), 1.0);
         tb_term(jb, trace_block<C>(ctx, j + 1, 0, 1), pair_ptr(y, ctx, 1, j + 1));
         rec_trace_blocks<C>(ctx, rec, {jb}, R);
@@ -1303,14 +1346,16 @@ void rec_apply_precond(Ctx& ctx, Rec& rec, const double2* x, int R, double2* y, 
     const long long ntr = ctx.ntr;
     const int ldc = padded_ldc(dbl, R);
     if (ldc > ctx.slot_cap) throw Error{HZ_ERR_ADMISSION, "too many columns for the layer workspace"};
-    // downward sweep (Algorithm 4)
-    rec_pairs_axpy(ctx, rec, pair_ptr(y, ctx, 0, 0), ntr, pair_ptr(x, ctx, 0, 0), ntr, -1.0, nullptr, 0, 0.0, 0, 1, R);
+    // downward sweep (Algorithm 4): y_j = G^j S_top y_{j-1} - x_j.  The slots of all the sweep's layers
+    // are cleared, and -x written, in one launch each before it; a step is then three launches
+    std::vector<int> inner;
+    for (int l = 1; l <= L - 2; ++l) inner.push_back(l);
+    rec_pairs_axpy(ctx, rec, pair_ptr(y, ctx, 0, 0), ntr, pair_ptr(x, ctx, 0, 0), ntr, -1.0, nullptr, 0, 0.0, 0, K, R);
+    rec_zero_slots<C>(ctx, rec, inner, ldc);
     for (int j = 1; j < K; ++j) {
         std::vector<int> one{j};
-        rec_zero_slots<C>(ctx, rec, one, ldc);
         rec_inject<C>(ctx, rec, {make_inject<C>(ctx, j, true, pair_ptr(y, ctx, 0, j - 1), ntr, ldc, 0)}, R);
         rec_subst<C>(ctx, rec, one, R, true, sparse_code(SP_TOP, SP_BOT));   // source on top, read at the bottom
-        rec_pairs_axpy(ctx, rec, pair_ptr(y, ctx, 0, j), ntr, pair_ptr(x, ctx, 0, j), ntr, -1.0, nullptr, 0, 0.0, 0, 1, R);
         std::vector<Extract<C>> ex;
         for (int pl = 0; pl < 2; ++pl)
             ex.push_back(make_extract<C>(ctx, j, true, pl, {0}, pair_ptr(y, ctx, 0, j) + pl * ctx.P, ntr, ldc, 1.0));
@@ -1338,14 +1383,13 @@ void rec_apply_precond(Ctx& ctx, Rec& rec, const double2* x, int R, double2* y, 
                 ex.push_back(make_extract<C>(ctx, j + 1, false, pl, {0}, pair_ptr(s, ctx, 1, j) + pl * ctx.P, ntr, ldc, -1.0));
         rec_extract<C>(ctx, rec, ex, R);
     }
-    // upward sweep (Algorithm 5)
-    rec_pairs_axpy(ctx, rec, pair_ptr(y, ctx, 1, K - 1), ntr, pair_ptr(s, ctx, 1, K - 1), ntr, -1.0, nullptr, 0, 0.0, 0, 1, R);
+    // upward sweep (Algorithm 5): y_j = G^{j+1} S_bot y_{j+1} - s_j
+    rec_pairs_axpy(ctx, rec, pair_ptr(y, ctx, 1, 0), ntr, pair_ptr(s, ctx, 1, 0), ntr, -1.0, nullptr, 0, 0.0, 0, K, R);
+    rec_zero_slots<C>(ctx, rec, inner, ldc);
     for (int j = K - 2; j >= 0; --j) {
         std::vector<int> one{j + 1};
-        rec_zero_slots<C>(ctx, rec, one, ldc);
         rec_inject<C>(ctx, rec, {make_inject<C>(ctx, j + 1, false, pair_ptr(y, ctx, 1, j + 1), ntr, ldc, 0)}, R);
         rec_subst<C>(ctx, rec, one, R, true, sparse_code(SP_BOT, SP_TOP));   // source at the bottom, read on top
-        rec_pairs_axpy(ctx, rec, pair_ptr(y, ctx, 1, j), ntr, pair_ptr(s, ctx, 1, j), ntr, -1.0, nullptr, 0, 0.0, 0, 1, R);
         std::vector<Extract<C>> ex;
         for (int pl = 0; pl < 2; ++pl)
             ex.push_back(make_extract<C>(ctx, j + 1, false, pl, {0}, pair_ptr(y, ctx, 1, j) + pl * ctx.P, ntr, ldc, 1.0));
@@ -1657,7 +1701,9 @@ void gmres_solve(Ctx& ctx, const double2* g, bool scale, int R, double2* u, cons
         k_scale_vec<<<gvec, TB, 0, st>>>(W.V, w, n, s.invb);
         HZ_CHECK_LAUNCH();
         if (!any_active()) break;
+        int used = 0;   // basis vectors of this cycle (a column's own count is at most this)
         for (int j = 0; j < m && total_it < o.max_iter; ++j) {
+            used = j + 1;
             matvec(W.V + (long long)j * vs, w);
             HZ_CUDA(cudaMemsetAsync(s.dots, 0, (size_t)R * (m + 1) * sizeof(double2), st));
             for (int pass = 0; pass < 2; ++pass) {  // classical Gram-Schmidt, twice
@@ -1680,7 +1726,7 @@ void gmres_solve(Ctx& ctx, const double2* g, bool scale, int R, double2* u, cons
         // x += V y for this cycle
         k_gmres_lsq<<<cdiv(R, 128), 128, 0, st>>>(s, R, m);
         HZ_CHECK_LAUNCH();
-        k_maxpy_plus<<<gvec, TB, 0, st>>>(W.V, vs, W.xs, n, m, s.y, m);
+        k_maxpy_plus<<<gvec, TB, 0, st>>>(W.V, vs, W.xs, n, used, s.y, m);
         HZ_CHECK_LAUNCH();
         if (!any_active() || total_it >= o.max_iter) break;
         // columns still active restart from their current iterate

@@ -119,8 +119,7 @@ template <int MODE, class C> __device__ inline const C* source_vec(const JobDev<
 
 template <class C, int CC, int MODE>
 __global__ void __launch_bounds__(256) k_subst(const Task* __restrict__ tasks,
-                                               const JobDev<C>* __restrict__ jobs, int ldc, int nchunks,
-                                               int KS) {
+                                               const JobDev<C>* __restrict__ jobs, int ldc, int nchunks) {
     constexpr int WC = CC >= 8 ? 8 : CC;  // warps along the columns
     constexpr int WK = 8 / WC;            // warps along the reduction dimension
     constexpr int NCT = CC / WC;          // columns per thread
@@ -137,14 +136,14 @@ __global__ void __launch_bounds__(256) k_subst(const Task* __restrict__ tasks,
     const int wc = warp % WC, wk = warp / WC;
     const int col0 = chunk * CC;
 
-    // reduction range of this task: [tk.pad_ (first tile), +KS) within the product's range
+    // reduction range of this task within the product's
     int kend;
     if (MODE == FA) kend = tk.tile + 1;
     else if (MODE == FB) kend = nd.own_t;
     else if (MODE == BA) kend = nd.upd_t;
     else kend = nd.own_t;
-    const int kt0 = tk.pad_;
-    const int kt1 = min(kend, kt0 + KS);
+    const int kt0 = tk.k0;
+    const int kt1 = kt0 + tk.klen;
 
     const C* vec = source_vec<MODE>(jb);
     const int* upd = jb.upd_idx + nd.upd_off;
@@ -235,8 +234,7 @@ __global__ void __launch_bounds__(256) k_subst(const Task* __restrict__ tasks,
 // on the way in for the transposed phases.
 template <int MODE>
 __global__ void __launch_bounds__(256, 4) k_subst64(const Task* __restrict__ tasks,
-                                                    const JobDev<float2>* __restrict__ jobs, int ldc, int nchunks,
-                                                    int KS) {
+                                                    const JobDev<float2>* __restrict__ jobs, int ldc, int nchunks) {
     constexpr int CC = 64;
     constexpr int MS = 34;                       // padded row length (complex) of the [k][row] tile
     constexpr int XP = CC + 2;                   // padded row length of the vector / output tile
@@ -256,8 +254,8 @@ __global__ void __launch_bounds__(256, 4) k_subst64(const Task* __restrict__ tas
     else if (MODE == FB) kend = nd.own_t;
     else if (MODE == BA) kend = nd.upd_t;
     else kend = nd.own_t;
-    const int kt0 = tk.pad_;
-    const int kt1 = min(kend, kt0 + KS);
+    const int kt0 = tk.k0;
+    const int kt1 = kt0 + tk.klen;
     const float2* vec = source_vec<MODE>(jb);
     const int* upd = jb.upd_idx + nd.upd_off;
 
@@ -346,24 +344,25 @@ void launch_level(const Batch& b, int h, int mode, int ldc, cudaStream_t st) {
     if constexpr (CC == 64 && sizeof(C) == 8) {
         const JobDev<float2>* j64 = (const JobDev<float2>*)b.d_jobs;
         switch (mode) {
-            case FA: k_subst64<FA><<<grid, 256, 0, st>>>(tasks, j64, ldc, nchunks, b.KS); break;
-            case FB: k_subst64<FB><<<grid, 256, 0, st>>>(tasks, j64, ldc, nchunks, b.KS); break;
-            case BA: k_subst64<BA><<<grid, 256, 0, st>>>(tasks, j64, ldc, nchunks, b.KS); break;
-            default: k_subst64<BB><<<grid, 256, 0, st>>>(tasks, j64, ldc, nchunks, b.KS); break;
+            case FA: k_subst64<FA><<<grid, 256, 0, st>>>(tasks, j64, ldc, nchunks); break;
+            case FB: k_subst64<FB><<<grid, 256, 0, st>>>(tasks, j64, ldc, nchunks); break;
+            case BA: k_subst64<BA><<<grid, 256, 0, st>>>(tasks, j64, ldc, nchunks); break;
+            default: k_subst64<BB><<<grid, 256, 0, st>>>(tasks, j64, ldc, nchunks); break;
         }
     } else {
         switch (mode) {
-            case FA: k_subst<C, CC, FA><<<grid, 256, 0, st>>>(tasks, jobs, ldc, nchunks, b.KS); break;
-            case FB: k_subst<C, CC, FB><<<grid, 256, 0, st>>>(tasks, jobs, ldc, nchunks, b.KS); break;
-            case BA: k_subst<C, CC, BA><<<grid, 256, 0, st>>>(tasks, jobs, ldc, nchunks, b.KS); break;
-            default: k_subst<C, CC, BB><<<grid, 256, 0, st>>>(tasks, jobs, ldc, nchunks, b.KS); break;
+            case FA: k_subst<C, CC, FA><<<grid, 256, 0, st>>>(tasks, jobs, ldc, nchunks); break;
+            case FB: k_subst<C, CC, FB><<<grid, 256, 0, st>>>(tasks, jobs, ldc, nchunks); break;
+            case BA: k_subst<C, CC, BA><<<grid, 256, 0, st>>>(tasks, jobs, ldc, nchunks); break;
+            default: k_subst<C, CC, BB><<<grid, 256, 0, st>>>(tasks, jobs, ldc, nchunks); break;
         }
     }
     HZ_CHECK_LAUNCH();
 }
 
 // One launch for the vectors of all layers (a memset node per layer costs a launch each: 2 x 16
-// of them per substitution at 16 layers).  16-byte stores, grid-stride; HBM/L2 write bound.
+// of them per substitution at 16 layers; clearing whole vectors took 31 of 943 ms of a 128^3 solve with
+// 32 columns, the rows of split reductions are a tenth of them).  16-byte stores, grid-stride; HBM/L2 write bound.
 __global__ void __launch_bounds__(256) k_zero(const ZeroDev* d) {
     const ZeroDev z = d[blockIdx.y];
     float4* p = (float4*)z.p;
@@ -420,9 +419,10 @@ void run_batch(const Batch& b, int ldc, int ncols, bool tc, int* flag, cudaStrea
             lt.done();
         }
     };
-    auto zero = [&](int which, int mode) {   // acc (0) / x (1) of every layer, before the launches of `mode`
-        LaunchTimer lt(pl, st, 0, 0.0, 0.0, mode, 0, (long long)b.vec_rows.size());
-        launch_zero(b.d_zero[which], (int)b.vec_rows.size(), b.zero_max, st);
+    auto zero = [&](int which, int mode) {   // rows of acc (0) / x (1) that the launches of `mode` add into
+        if (b.zero_n[which] == 0) return;
+        LaunchTimer lt(pl, st, 0, 0.0, 0.0, mode, 0, b.zero_n[which]);
+        launch_zero(b.d_zero[which], b.zero_n[which], b.zero_max, st);
         lt.done();
     };
     if (has_m21<C>) {   // FA and BB hold the nodes of all levels at index 0
@@ -447,8 +447,10 @@ void run_batch(const Batch& b, int ldc, int ncols, bool tc, int* flag, cudaStrea
 void launch_zero(const ZeroDev* d, int n, long long max_bytes, cudaStream_t st) {
     if (n <= 0 || max_bytes <= 0) return;
     const unsigned gx = (unsigned)std::max<long long>(1, std::min<long long>(cdiv(max_bytes / 16, 1024), 1216));
-    k_zero<<<dim3(gx, (unsigned)n), 256, 0, st>>>(d);
-    HZ_CHECK_LAUNCH();
+    for (int i = 0; i < n; i += 65535) {
+        k_zero<<<dim3(gx, (unsigned)std::min(n - i, 65535)), 256, 0, st>>>(d + i);
+        HZ_CHECK_LAUNCH();
+    }
 }
 
 int chunk_cols(bool is_double, int ncols) {
@@ -661,9 +663,18 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
             b.lvl_flops[k][mode].assign(H, 0.0);
         }
     auto add_tasks = [&](std::vector<Task>& out, int j, int nid, int tile, int k0, int k1, int ks) {
-        if (k1 <= k0) { out.push_back(Task{j, nid, tile, k0}); return; }
-        for (int k = k0; k < k1; k += ks) out.push_back(Task{j, nid, tile, k});
+        if (k1 >= 65536) throw Error{HZ_ERR_ARG, "node product too long"};
+        if (k1 <= k0) { out.push_back(Task{j, nid, tile, (unsigned short)k0, 0}); return; }
+        for (int k = k0; k < k1; k += std::min(ks, k1 - k))
+            out.push_back(Task{j, nid, tile, (unsigned short)k, (unsigned short)std::min(ks, k1 - k)});
     };
+    // M21: FA and BB of all levels share a launch, which needs no split to fill the GPU, only to keep its
+    // longest reductions from trailing: 16 tiles or the update products' depth, the root in two.  Whole
+    // reductions are stored; only the rows of split ones have to be cleared beforehand.
+    auto diag_ks = [&](const Node& nd, int ks) {
+        return std::min(std::max(ks, 16), nd.parent < 0 ? std::max(1, (nd.own_t + 1) / 2) : 1 << 30);
+    };
+    std::vector<ZeroDev> zero_rows[2];   // acc, x
     for (int j = 0; j < (int)layers.size(); ++j) {
         const Layer& ly = ctx.layers[layers[j]];
         const Shape& sh = ctx.shapes[ly.shape];
@@ -700,6 +711,8 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
                     const bool fwd = mode == FA || mode == FB;
                     const int out_t = mode == 1 ? nd.upd_t : nd.own_t;
                     const bool on_tc = tc && tc_node(mode, nd, b.min_t);
+                    const bool diag = m21 && (mode == 0 || mode == 3);
+                    const int ks_tc = diag ? diag_ks(nd, b.KS_tc) : b.KS_tc, ks = diag ? diag_ks(nd, KS) : KS;
                     int nact = 0;
                     if (m21 && mode == 2 && nd.nupd == 0) continue;   // the root has nothing to gather
                     // M21: FA and BB of every level go in one launch each
@@ -717,21 +730,25 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
                             prods.push_back({mode, h, jq, nid});
                         } else if (on_tc) {
                             for (int t = 0; t < out_t; t += 4) {
-                                if (mode == 0) add_tasks(quads[0][hl], jq, nid, t, 0, std::min(t + 4, nd.own_t), b.KS_tc);
-                                if (mode == 1) add_tasks(quads[1][hl], jq, nid, t, 0, nd.own_t, b.KS_tc);
-                                if (mode == 2) add_tasks(quads[2][hl], jq, nid, t, 0, nd.upd_t, b.KS_tc);
-                                if (mode == 3) add_tasks(quads[3][hl], jq, nid, t, t, nd.own_t, b.KS_tc);
+                                if (mode == 0) add_tasks(quads[0][hl], jq, nid, t, 0, std::min(t + 4, nd.own_t), ks_tc);
+                                if (mode == 1) add_tasks(quads[1][hl], jq, nid, t, 0, nd.own_t, ks_tc);
+                                if (mode == 2) add_tasks(quads[2][hl], jq, nid, t, 0, nd.upd_t, ks_tc);
+                                if (mode == 3) add_tasks(quads[3][hl], jq, nid, t, t, nd.own_t, ks_tc);
                             }
                         } else {
                             for (int t = 0; t < out_t; ++t) {
-                                if (mode == 0) add_tasks(lists[0][hl], jq, nid, t, 0, t + 1, KS);      // FA: Linv row tile t
-                                if (mode == 1) add_tasks(lists[1][hl], jq, nid, t, 0, nd.own_t, KS);   // FB: L21 row tile t
-                                if (mode == 2) add_tasks(lists[2][hl], jq, nid, t, 0, nd.upd_t, KS);   // BA (>= 1 task)
-                                if (mode == 3) add_tasks(lists[3][hl], jq, nid, t, t, nd.own_t, KS);   // BB
+                                if (mode == 0) add_tasks(lists[0][hl], jq, nid, t, 0, t + 1, ks);      // FA: Linv row tile t
+                                if (mode == 1) add_tasks(lists[1][hl], jq, nid, t, 0, nd.own_t, ks);   // FB: L21 row tile t
+                                if (mode == 2) add_tasks(lists[2][hl], jq, nid, t, 0, nd.upd_t, ks);   // BA (>= 1 task)
+                                if (mode == 3) add_tasks(lists[3][hl], jq, nid, t, t, nd.own_t, ks);   // BB
                             }
                         }
                     }
                     if (nact == 0) continue;
+                    if (diag && nd.own_t > (on_tc ? ks_tc : ks)) {
+                        C* v = (C*)(mode == 0 ? ctx.slot_x[layers[j]] : ctx.slot_acc[layers[j]]) + (long long)nd.own0 * ldc;
+                        zero_rows[mode == 0].push_back({v, (long long)nd.nown * ldc * (long long)sizeof(C)});
+                    }
                     // stored factor entries this product reads (triangular L^{-1} or L21): once
                     // algorithmically, however many column blocks use them
                     const double ent = (mode == FA || mode == BB) ? (double)nd.nown * (nd.nown + 1) / 2.0
@@ -745,22 +762,11 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
     // round-robin, and every kernel then ends a launch on short items
     for (int mode = 0; mode < 4; ++mode)
         for (int h = 0; h < H; ++h) {
-            auto sort_items = [&](std::vector<Task>& v, int rows, int ks) {
-                auto red_len = [&](const Task& tk) {
-                    const Node& nd = ctx.shapes[ctx.layers[layers[tk.job / nblk]].shape].nodes[tk.node];
-                    const int kend = mode == 0 ? std::min(tk.tile + rows, nd.own_t) : (mode == 2 ? nd.upd_t : nd.own_t);
-                    return std::min(kend, tk.pad_ + std::min(ks, 1 << 28)) - tk.pad_;
-                };
-                std::vector<std::pair<int, int>> order(v.size());
-                for (int i = 0; i < (int)v.size(); ++i) order[i] = {-red_len(v[i]), i};
-                std::sort(order.begin(), order.end());
-                std::vector<Task> sorted;
-                sorted.reserve(v.size());
-                for (auto& o : order) sorted.push_back(v[o.second]);
-                v.swap(sorted);
+            auto sort_items = [&](std::vector<Task>& v) {
+                std::stable_sort(v.begin(), v.end(), [](const Task& x, const Task& y) { return x.klen > y.klen; });
             };
-            sort_items(quads[mode][h], 4, b.KS_tc);
-            if (m21) sort_items(lists[mode][h], 1, KS);
+            sort_items(quads[mode][h]);
+            if (m21) sort_items(lists[mode][h]);
         }
     std::vector<Task> all;
     for (int mode = 0; mode < 4; ++mode) {
@@ -811,13 +817,13 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
             }
     if (stream) build_stream(ctx, layers, prods, H, b.plan);
     for (int w = 0; w < 2; ++w) {
-        std::vector<ZeroDev> zd;
-        for (size_t j = 0; j < b.vec_ptrs.size(); ++j) {
-            const long long bytes = b.vec_rows[j] * ldc * (long long)sizeof(C);
-            zd.push_back({w ? b.vec_ptrs[j].second : b.vec_ptrs[j].first, bytes});
-            b.zero_max = std::max(b.zero_max, bytes);
-        }
-        HZ_CUDA(cudaMalloc(&b.d_zero[w], zd.size() * sizeof(ZeroDev)));
+        std::vector<ZeroDev>& zd = zero_rows[w];
+        if (!m21)
+            for (size_t j = 0; j < b.vec_ptrs.size(); ++j)
+                zd.push_back({w ? b.vec_ptrs[j].second : b.vec_ptrs[j].first, b.vec_rows[j] * ldc * (long long)sizeof(C)});
+        for (const ZeroDev& z : zd) b.zero_max = std::max(b.zero_max, z.bytes);
+        b.zero_n[w] = (int)zd.size();
+        HZ_CUDA(cudaMalloc(&b.d_zero[w], std::max<size_t>(1, zd.size()) * sizeof(ZeroDev)));
         HZ_CUDA(cudaMemcpyAsync(b.d_zero[w], zd.data(), zd.size() * sizeof(ZeroDev), cudaMemcpyHostToDevice, ctx.stream));
         HZ_CUDA(cudaStreamSynchronize(ctx.stream));
     }

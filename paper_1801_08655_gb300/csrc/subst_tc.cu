@@ -108,7 +108,7 @@ struct Item {
 };
 
 template <int NT, int MODE>
-__device__ inline Item decode(const Task* tasks, const JobDev<float2>* jobs, long long item, int nchunks, int KS) {
+__device__ inline Item decode(const Task* tasks, const JobDev<float2>* jobs, long long item, int nchunks) {
     Item it;
     const Task tk = tasks[item / nchunks];
     it.jb = jobs[tk.job];
@@ -119,11 +119,11 @@ __device__ inline Item decode(const Task* tasks, const JobDev<float2>* jobs, lon
     it.nout_t = (MODE == FB) ? nd.upd_t : nd.own_t;
     it.nrows_out = (MODE == FB) ? nd.nupd : nd.nown;
     it.nrows_k = (MODE == BA) ? nd.nupd : nd.nown;
-    it.kbeg = tk.pad_;
+    it.kbeg = tk.k0;
     const int kfull0 = (MODE == BB) ? it.o0 : 0;
     const int kfull1 = (MODE == FA) ? min(it.o0 + 4, nd.own_t) : ((MODE == BA) ? nd.upd_t : nd.own_t);
-    it.kend = min(kfull1, it.kbeg + KS);
-    it.nst = max(0, it.kend - it.kbeg) * 2;
+    it.kend = it.kbeg + tk.klen;
+    it.nst = tk.klen * 2;
     it.unique = it.kbeg == kfull0 && it.kend == kfull1 && MODE != FB && MODE != BA;
     return it;
 }
@@ -294,7 +294,7 @@ template <int NT> struct OneLayout {
 
 template <int NT, int MODE, int SPLIT>
 __global__ void __launch_bounds__(OneLayout<NT>::NTHREADS, 1)
-k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jobs, int ldc, int nchunks, int KS,
+k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jobs, int ldc, int nchunks,
            int* flag, long long polls) {
     using RG = Ring<NT>;
     using LY = OneLayout<NT>;
@@ -313,7 +313,7 @@ k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jo
     volatile int* abort = (volatile int*)tptr + 1;
     volatile int* committed = (volatile int*)tptr + 2;   // stages whose MMAs were committed
 
-    const Item it = decode<NT, MODE>(tasks, jobs, blockIdx.x, nchunks, KS);
+    const Item it = decode<NT, MODE>(tasks, jobs, blockIdx.x, nchunks);
     const int t = threadIdx.x, w = t >> 5, l = t & 31;
     const int nst = it.nst;
     const int mma_warp = (NLOAD + NCONV) / 32;
@@ -466,7 +466,7 @@ template <int NT> struct PLayout {
 
 template <int NT, int MODE, int SPLIT>
 __global__ void __launch_bounds__(PLayout<NT>::NTHREADS, 1)
-k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jobs, int ldc, int nchunks, int KS,
+k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jobs, int ldc, int nchunks,
             long long nitems, int* flag, long long polls) {
     using RG = Ring<NT>;
     using LY = PLayout<NT>;
@@ -523,13 +523,13 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
         Item cur;
         Vrows<NT> rows;
         if (item < nitems) {
-            cur = decode<NT, MODE>(tasks, jobs, item, nchunks, KS);
+            cur = decode<NT, MODE>(tasks, jobs, item, nchunks);
             rows = stage_rows<NT, MODE>(cur, 0, t);
         }
         for (; item < nitems && ok; item += gridDim.x) {
             const long long nxt_item = item + gridDim.x;
             Item nxt = cur;
-            if (nxt_item < nitems) nxt = decode<NT, MODE>(tasks, jobs, nxt_item, nchunks, KS);
+            if (nxt_item < nitems) nxt = decode<NT, MODE>(tasks, jobs, nxt_item, nchunks);
             for (int s = 0; s < cur.nst && ok; ++s, ++gs) {
                 const int slot = (int)(gs % RD);
                 const long long use = gs / RD;
@@ -549,10 +549,10 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
         // ------------------------------------------------------------ converters
         const int ct = t - NLOAD;
         long long gs = 0;
-        int nst_next = blockIdx.x < nitems ? decode<NT, MODE>(tasks, jobs, blockIdx.x, nchunks, KS).nst : 0;
+        int nst_next = blockIdx.x < nitems ? decode<NT, MODE>(tasks, jobs, blockIdx.x, nchunks).nst : 0;
         for (long long item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
             const int nst = nst_next;   // decoded one item ahead
-            if (item + gridDim.x < nitems) nst_next = decode<NT, MODE>(tasks, jobs, item + gridDim.x, nchunks, KS).nst;
+            if (item + gridDim.x < nitems) nst_next = decode<NT, MODE>(tasks, jobs, item + gridDim.x, nchunks).nst;
             for (int s = 0; s < nst && ok; ++s, ++gs) {
                 const int slot = (int)(gs % RD), cb = (int)(gs & 1);
                 const long long use = gs / RD, cuse = gs >> 1;
@@ -570,10 +570,10 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
         if (l == 0) {
             long long gs = 0;
             int nit = 0;  // items of this block so far
-            int nst_next = blockIdx.x < nitems ? decode<NT, MODE>(tasks, jobs, blockIdx.x, nchunks, KS).nst : 0;
+            int nst_next = blockIdx.x < nitems ? decode<NT, MODE>(tasks, jobs, blockIdx.x, nchunks).nst : 0;
             for (long long item = blockIdx.x; item < nitems && ok; item += gridDim.x, ++nit) {
                 const int nst = nst_next;   // decoded one item ahead
-                if (item + gridDim.x < nitems) nst_next = decode<NT, MODE>(tasks, jobs, item + gridDim.x, nchunks, KS).nst;
+                if (item + gridDim.x < nitems) nst_next = decode<NT, MODE>(tasks, jobs, item + gridDim.x, nchunks).nst;
                 const int b = nit & 1;
                 if (nit >= 2) ok = mbar_wait(smem_u32(acc_empty + b), (uint32_t)(((nit >> 1) - 1) & 1), abort, polls);
                 if (!ok) break;
@@ -607,7 +607,7 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
         const int r4 = l >> 3, p = l & 7;   // write phase: row within a group of 4, column pair
         int nit = 0;
         for (long long item = blockIdx.x; item < nitems && ok; item += gridDim.x, ++nit) {
-            const Item it = decode<NT, MODE>(tasks, jobs, item, nchunks, KS);
+            const Item it = decode<NT, MODE>(tasks, jobs, item, nchunks);
             const int b = nit & 1;
             // this lane's row descriptor, shuffled to the writing lanes below
             const long long my_base = row_base<MODE>(it, 32 * q4 + l, ldc);
@@ -683,7 +683,7 @@ void launch_one(const Batch& b, const Task* tasks, long long n, const JobDev<flo
         }
         const long long grid = std::min<long long>(nitems, sm_count());
         k_subst_tcp<NT, MODE, SPLIT><<<(unsigned)grid, PLayout<NT>::NTHREADS, PLayout<NT>::TOTAL, st>>>(
-            tasks, jobs, ldc, nchunks, b.KS_tc, nitems, flag, b.wait_polls);
+            tasks, jobs, ldc, nchunks, nitems, flag, b.wait_polls);
     } else {
         static bool attr = false;
         if (!attr) {
@@ -692,7 +692,7 @@ void launch_one(const Batch& b, const Task* tasks, long long n, const JobDev<flo
             attr = true;
         }
         k_subst_tc<NT, MODE, SPLIT><<<(unsigned)nitems, OneLayout<NT>::NTHREADS, OneLayout<NT>::TOTAL, st>>>(
-            tasks, jobs, ldc, nchunks, b.KS_tc, flag, b.wait_polls);
+            tasks, jobs, ldc, nchunks, flag, b.wait_polls);
     }
     HZ_CHECK_LAUNCH();
 }
