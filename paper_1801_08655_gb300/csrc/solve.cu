@@ -581,7 +581,10 @@ void ensure_tuned(Ctx& ctx, const std::vector<int>& layers, int ncols, int split
         std::vector<int> mts{2};
         if (ctx.tc_min_tiles < 8 && ctx.tc_min_tiles != 2) mts.push_back(ctx.tc_min_tiles);
         for (int mt : mts) {
-            for (int kstc : {2, 4, 8, 16, 1 << 30}) cands.push_back({8, cc0, 1, kstc, mt, 1});
+            // factors from FP64: the per-item kernel alone, whose hi x lo terms have accumulators of their
+            // own at every width (a 40^3 layer solve on 64 columns 2.5e-6 off, 1.0e-5 without)
+            if (ctx.prec == HZ_PREC_MIXED)
+                for (int kstc : {2, 4, 8, 16, 1 << 30}) cands.push_back({8, cc0, 1, kstc, mt, 1});
             for (int kstc : {4, 1 << 30}) cands.push_back({8, cc0, 1, kstc, mt, 0});
         }
     }

@@ -21,7 +21,7 @@
 //                       buffer (masked rows / absent tiles zero-filled by the copy), completion
 //                       signalled with cp.async.mbarrier.arrive;
 //   8 converter warps : raw -> split hi/lo TF32 operands in the K-major core-matrix layout
-//                       (no swizzle), 16-byte stores;
+//                       (no swizzle), 16-byte stores, or the factor's in tensor memory;
 //   1 MMA warp        : one thread issues the MMAs of a stage and commits them to the mbarrier
 //                       that releases the converted buffer.
 // Two kernels share these stages:
@@ -57,9 +57,8 @@ enum { FA = 0, FB = 1, BA = 2, BB = 3 };
 // operands per stage, which does not fit beside a two-deep raw ring, and fills N = 128 as it is.
 // The room that narrow tiles leave goes to the raw ring: the factor stream, 16 KB per stage
 // whatever NT is, binds them, and every further stage in flight covers memory latency.
-// Measured: a 32-column block of a 128^3 layer 3.10 ms on the CUDA cores, 1.68 here (115-120
-// TFLOP/s on the upper levels; about 1200 shared-memory cycles a stage allow 140); 64 columns, 64^3,
-// 8 layers: 3.98 ms with N = 64 MMAs on a two-deep ring, 2.80 in the wide form.
+// Measured: a 32-column block of a 128^3 layer 3.10 ms on the CUDA cores, 1.68 in the wide form; 64
+// columns, 64^3, 8 layers: 3.98 ms with N = 64 MMAs on a two-deep ring, 2.80 in the wide form.
 template <int NT> struct Ring {
     static constexpr bool WIDE = NT <= 64;
     static constexpr int A_MAT = MR * KC * 4;            // one real operand matrix (8 KB)
@@ -76,10 +75,10 @@ template <int NT> struct Ring {
 // Columns of one accumulator set: real and imaginary part, and (SEP) the hi x lo terms' own.
 template <int NT, int SPLIT, bool SEP> constexpr int acc_cols = (SEP && SPLIT == 3) ? 4 * NT : 2 * NT;
 
-template <int NT, int SPLIT, bool SEP>
-__device__ __forceinline__ void mma_item_stage(uint32_t conv, uint32_t tm, bool first) {
-    static_assert(!Ring<NT>::WIDE || SEP, "the wide form keeps the hi x lo terms apart");
-    if constexpr (Ring<NT>::WIDE) mma_stage_wide<NT, SPLIT>(conv, tm, first);
+template <int NT, int SPLIT, bool SEP, bool TA>
+__device__ __forceinline__ void mma_item_stage(uint32_t conv, uint32_t tm, bool first, uint32_t ta) {
+    static_assert(Ring<NT>::WIDE || !TA, "the factor operand is in tensor memory in the wide form only");
+    if constexpr (Ring<NT>::WIDE) mma_stage_wide<NT, SPLIT, SEP, TA>(conv, tm, first, ta);
     else mma_stage<NT, SPLIT, SEP>(conv, tm, tm + NT, first);
 }
 
@@ -148,39 +147,64 @@ __device__ inline Vrows<NT> stage_rows(const Item& it, int s, int t) {
     return v;
 }
 
-// Loader part of stage s of an item: the four factor tiles' 16-column halves and 16 vector rows.
-template <int NT, int MODE>
-__device__ inline void load_stage(unsigned char* rb, const Item& it, int s, int ldc, int t, const Vrows<NT>& vr) {
-    using RG = Ring<NT>;
-    constexpr bool TR = (MODE == BA || MODE == BB);  // factor tiles used transposed
-    const NodeDev& nd = it.nd;
-    const int kt = it.kbeg + (s >> 1), hk = s & 1;
-    for (int c = t; c < 1024; c += NLOAD) {     // factor tiles: 1024 chunks of 16 bytes
-        const int oi = c >> 8, q = c & 255;
-        const int o = it.o0 + oi;
-        bool exists = o < it.nout_t;
-        if (MODE == FA) exists = exists && kt <= o;
-        if (MODE == BB) exists = exists && kt >= o;
-        long long toff = 0;
-        if (exists) {
+// The four factor tiles of an item's current reduction tile, as one loader thread copies them: its
+// first 16 bytes of each (8 per stage: 4 tiles x 2, 2 KB apart as stored, 16 columns apart where used
+// transposed).  Pointers advance from tile to tile; forming every copy's address anew (triangular
+// index, 64-bit products) kept a loader warp at some 230 instructions a stage, which bound narrow tiles.
+template <int MODE> struct TilePtrs {
+    static constexpr bool TR = (MODE == BA || MODE == BB);
+    const char* p[4];
+    int kt, o0, nout_t;
+    long long step;   // bytes to the next reduction tile (BB: of the first one on)
+
+    __device__ __forceinline__ void init(const Item& it, int t) {
+        const NodeDev& nd = it.nd;
+        kt = it.kbeg;
+        o0 = it.o0;
+        nout_t = it.nout_t;
+        const int thr = TR ? (t >> 3) * 256 + (t & 7) * 16 : t * 16;
+#pragma unroll
+        for (int oi = 0; oi < 4; ++oi) {
+            const int o = o0 + oi;
+            long long toff;
             if (MODE == FA) toff = nd.linv_off + tri_idx(o, kt);
             else if (MODE == FB) toff = nd.l21_off + (long long)o * nd.own_t + kt;
             else if (MODE == BA) toff = nd.l21_off + (long long)kt * nd.own_t + o;
             else toff = nd.linv_off + tri_idx(kt, o);
+            p[oi] = (const char*)(it.jb.fac + toff * TILE2) + thr;
         }
-        const float2* tl = it.jb.fac + toff * TILE2;
-        uint32_t dst;
-        const float2* src;
-        if (!TR) {
-            dst = smem_u32(rb + oi * 4096 + q * 16);
-            src = tl + hk * KC * 32 + q * 2;
-        } else {
-            const int r = q >> 3, j = q & 7;
-            dst = smem_u32(rb + oi * 32 * TROW + r * TROW + j * 16);
-            src = tl + 32 * r + hk * KC + j * 2;
-        }
-        cp16(dst, exists ? (const void*)src : (const void*)it.jb.fac, exists ? 16 : 0);
+        step = (MODE == BA ? (long long)nd.own_t : MODE == BB ? (long long)kt + 1 : 1LL) * (TILE2 * 8);
     }
+    __device__ __forceinline__ void next() {
+#pragma unroll
+        for (int oi = 0; oi < 4; ++oi) p[oi] += step;
+        ++kt;
+        if (MODE == BB) step += TILE2 * 8;
+    }
+    __device__ __forceinline__ bool exists(int oi) const {
+        const int o = o0 + oi;
+        return o < nout_t && (MODE != FA || kt <= o) && (MODE != BB || kt >= o);
+    }
+};
+
+// Loader part of stage s of an item: the four factor tiles' 16-column halves and 16 vector rows.
+template <int NT, int MODE>
+__device__ inline void load_stage(unsigned char* rb, const Item& it, TilePtrs<MODE>& tp, int s, int ldc, int t,
+                                  const Vrows<NT>& vr) {
+    using RG = Ring<NT>;
+    constexpr bool TR = (MODE == BA || MODE == BB);  // factor tiles used transposed
+    const int hk = s & 1;
+    const uint32_t dst = smem_u32(rb) + (TR ? (t >> 3) * TROW + (t & 7) * 16 : t * 16);
+#pragma unroll
+    for (int oi = 0; oi < 4; ++oi) {   // factor tiles: 1024 chunks of 16 bytes
+        const bool ex = tp.exists(oi);
+        const char* src = ex ? tp.p[oi] + hk * (TR ? KC * 8 : KC * 32 * 8) : (const char*)it.jb.fac;
+        const int n = ex ? 16 : 0;
+        constexpr int DT = TR ? 32 * TROW : 4096;
+        cp16(dst + oi * DT, src, n);
+        cp16(dst + oi * DT + (TR ? 16 * TROW : 2048), ex ? src + (TR ? 16 * 256 : 2048) : src, n);
+    }
+    if (hk) tp.next();
     const float2* vec = MODE == BB ? it.jb.x : it.jb.acc;
 #pragma unroll
     for (int i = 0; i < KC * NT / 2 / NLOAD; ++i) {  // vector rows: KC x NT, raw [k][n]
@@ -192,12 +216,45 @@ __device__ inline void load_stage(unsigned char* rb, const Item& it, int s, int 
     }
 }
 
-// Converter part of a stage: raw -> hi (and lo) TF32 operands.
-template <int NT, int MODE, int SPLIT>
-__device__ inline void convert_stage(const unsigned char* rb, unsigned char* cv, int ct) {
+// Converter part of a stage: raw -> hi (and lo) TF32 operands, the vectors in shared memory, the factor
+// there or (TA) in tensor memory from column ta on: converter warp w writes the 32 lanes (rows) of tile
+// w % 4 that its place in the block gives it access to, 8 of the 16 columns of each matrix.
+// The stage is NTHR threads' work.
+template <int NT, int MODE, int SPLIT, bool TA, int NTHR>
+__device__ inline void convert_stage(const unsigned char* rb, unsigned char* cv, int ct, uint32_t ta) {
     using RG = Ring<NT>;
     constexpr bool TR = (MODE == BA || MODE == BB);
-    for (int id = ct; id < MR * 4; id += NCONV) {   // factor operand: 128 rows x 16 k, (row, 4 consecutive k)
+    if constexpr (TA) {
+        static_assert(NLOAD % 128 == 0 && NTHR == 128, "converter warp w must have warp index 4 n + w");
+        const int oi = ct >> 5, r = ct & 31;
+#pragma unroll
+        for (int kh = 0; kh < 2; ++kh) {
+            float re[8], im[8];
+            if (!TR) {
+                const float2* src = (const float2*)(rb + oi * 4096) + 8 * kh * 32 + r;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) { const float2 a = src[j * 32]; re[j] = a.x; im[j] = a.y; }
+            } else {
+                const float4* src = (const float4*)(rb + oi * 32 * TROW + r * TROW + kh * 64);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float4 a = src[j];
+                    re[2 * j] = a.x; im[2 * j] = a.y; re[2 * j + 1] = a.z; im[2 * j + 1] = a.w;
+                }
+            }
+            float hi[8];
+            const uint32_t col = ta + ((uint32_t)(32 * oi) << 16) + 8 * kh;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) { hi[j] = tf32_hi(re[j]); re[j] -= hi[j]; }
+            tmem_st8(col, hi);
+            if (SPLIT == 3) tmem_st8(col + KC, re);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) { hi[j] = tf32_hi(im[j]); im[j] -= hi[j]; }
+            tmem_st8(col + 2 * KC, hi);
+            if (SPLIT == 3) tmem_st8(col + 3 * KC, im);
+        }
+    }
+    for (int id = ct; !TA && id < MR * 4; id += NTHR) {   // factor operand: 128 rows x 16 k, (row, 4 consecutive k)
         const int row = id & 127, kq = id >> 7;
         const int oi = row >> 5, r = row & 31;
         float re[4], im[4];
@@ -222,7 +279,7 @@ __device__ inline void convert_stage(const unsigned char* rb, unsigned char* cv,
             *(float4*)(cv + 3 * RG::A_MAT + off) = make_float4(im[0] - ih.x, im[1] - ih.y, im[2] - ih.z, im[3] - ih.w);
         }
     }
-    for (int id = ct; id < NT * 4; id += NCONV) {   // vector operand: NT rows x 16 k
+    for (int id = ct; id < NT * 4; id += NTHR) {   // vector operand: NT rows x 16 k
         const int n = id % NT, kq = id / NT;
         const float2* src = (const float2*)(rb + RG::RAW_A);
         float re[4], im[4];
@@ -231,7 +288,7 @@ __device__ inline void convert_stage(const unsigned char* rb, unsigned char* cv,
         float4 rh, ih;
         rh.x = tf32_hi(re[0]); rh.y = tf32_hi(re[1]); rh.z = tf32_hi(re[2]); rh.w = tf32_hi(re[3]);
         ih.x = tf32_hi(im[0]); ih.y = tf32_hi(im[1]); ih.z = tf32_hi(im[2]); ih.w = tf32_hi(im[3]);
-        const int off = 4 * RG::A_MAT + coff(n, 4 * kq);
+        const int off = (TA ? 0 : 4 * RG::A_MAT) + coff(n, 4 * kq);
         const float4 rl = make_float4(re[0] - rh.x, re[1] - rh.y, re[2] - rh.z, re[3] - rh.w);
         const float4 il = make_float4(im[0] - ih.x, im[1] - ih.y, im[2] - ih.z, im[3] - ih.w);
         if (RG::WIDE) {
@@ -251,6 +308,10 @@ __device__ inline void convert_stage(const unsigned char* rb, unsigned char* cv,
                 *(float4*)(cv + off + 3 * RG::X_MAT) = il;
             }
         }
+    }
+    if constexpr (TA) {
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     }
 }
 
@@ -342,12 +403,14 @@ k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jo
 
     if (t < NLOAD) {
         Vrows<NT> rows = stage_rows<NT, MODE>(it, 0, t);
+        TilePtrs<MODE> tp;
+        tp.init(it, t);
         for (int s = 0; s < nst && ok; ++s) {
             const int slot = s % RD, use = s / RD;
             const Vrows<NT> next = stage_rows<NT, MODE>(it, s + 1, t);   // looked up ahead
             if (s >= RD) ok = mbar_wait(smem_u32(raw_empty + slot), (uint32_t)((use - 1) & 1), abort, polls);
             if (!ok) break;
-            load_stage<NT, MODE>(raw + slot * RG::RAW, it, s, ldc, t, rows);
+            load_stage<NT, MODE>(raw + slot * RG::RAW, it, tp, s, ldc, t, rows);
             cp_async_arrive(raw_full + slot);
             rows = next;
         }
@@ -365,7 +428,7 @@ k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jo
             ok = mbar_wait(smem_u32(raw_full + slot), (uint32_t)(use & 1), abort, polls);
             if (ok && s >= 2) ok = mbar_wait(smem_u32(conv_empty + cb), (uint32_t)((cuse - 1) & 1), abort, polls);
             if (!ok) break;
-            convert_stage<NT, MODE, SPLIT>(raw + slot * RG::RAW, conv + cb * RG::CONV, ct);
+            convert_stage<NT, MODE, SPLIT, false, NCONV>(raw + slot * RG::RAW, conv + cb * RG::CONV, ct, 0);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_arrive(raw_empty + slot);
             mbar_arrive(conv_full + cb);
@@ -376,7 +439,7 @@ k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jo
             ok = mbar_wait(smem_u32(conv_full + cb), (uint32_t)(use & 1), abort, polls);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            mma_item_stage<NT, SPLIT, true>(smem_u32(conv + cb * RG::CONV), tmem, s == 0);
+            mma_item_stage<NT, SPLIT, true, false>(smem_u32(conv + cb * RG::CONV), tmem, s == 0, 0);
             mma_commit(conv_empty + cb);
             *committed = s + 1;
         }
@@ -451,17 +514,29 @@ k_subst_tc(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ jo
 // ------------------------------------------------------------------------------------------
 // k_subst_tcp: persistent, one block per SM
 // ------------------------------------------------------------------------------------------
+// The wide tiles (NT <= 64) hold the factor operand in tensor memory: the converters write it there from
+// registers, so that of the shared-memory traffic of a stage (NT = 32: 16 KB copied in, 16 read back, 32
+// of operands written, 48 + 24 read by the MMAs) the factor's 80 KB of operands go.  The columns that the
+// accumulators leave are its ring.  NT = 128 has none left: its two buffers take all 512 columns.
+// Measured (128^3 layer, 32 columns / 64^3, 8 layers, 64 columns): operands in shared memory 1.68 / 2.80
+// ms, in tensor memory 1.58 / 2.45, with two converter groups 1.53 / 2.33, row look-ups two stages ahead
+// and integer rounding 1.48 / 2.24, running tile pointers 1.40 / 2.13; 128 columns (64^3, M_pol) 9.69 ->
+// 8.17 from the last three.  A third of the MMAs would save 15 %: the instruction streams of the loaders
+// and converters bind the narrow tiles, the shared-memory banks NT = 128.
 template <int NT> struct PLayout {
     using RG = Ring<NT>;
+    static constexpr bool TA = RG::WIDE;
+    // the hi x lo terms' own accumulators fit beside the factor ring at NT = 32
+    static constexpr bool SEP = NT == 32;
+    static constexpr int CD = NT == 32 ? 4 : NT == 64 ? 3 : 2;     // converted operands' ring depth
+    static constexpr int RD = NT == 32 ? 6 : NT == 64 ? 4 : 2;     // raw ring depth
+    static constexpr int CONV = TA ? 6 * RG::X_MAT : RG::CONV;
     static constexpr int NEPI = 128;                       // epilogue threads (4 warps)
     static constexpr int NTHREADS = NLOAD + NCONV + 32 + NEPI;
     static constexpr int EP = 18;                          // staging pitch (complex) of a 32 x 16 chunk
-    static constexpr int STG_OFF = RG::BYTES;              // 4 warps x 32 rows x EP complex
+    static constexpr int STG_OFF = CD * CONV + RD * RG::RAW;   // 4 warps x 32 rows x EP complex
     static constexpr int BAR_OFF = STG_OFF + 4 * 32 * EP * 8;
-    static constexpr int TOTAL = BAR_OFF + (2 * RG::RD + 8) * 8 + 16;
-    // two accumulator buffers; at NT = 128 they take all 512 columns, with no room for the hi x lo
-    // terms' own accumulators
-    static constexpr bool SEP = NT <= 64;
+    static constexpr int TOTAL = BAR_OFF + (2 * RD + 2 * CD + 4) * 8 + 16;
 };
 
 template <int NT, int MODE, int SPLIT>
@@ -471,16 +546,19 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
     using RG = Ring<NT>;
     using LY = PLayout<NT>;
     extern __shared__ __align__(1024) unsigned char smem[];
-    unsigned char* conv = smem;                  // [2][CONV]
-    unsigned char* raw = smem + 2 * RG::CONV;    // [RD][RAW]
-    constexpr int RD = RG::RD;
-    constexpr bool SEP = LY::SEP;
-    constexpr int BCOLS = acc_cols<NT, SPLIT, SEP>, TCOLS = 2 * BCOLS;   // one buffer, both
+    constexpr int RD = LY::RD, CD = LY::CD, CGRP = NCONV / 2;
+    constexpr bool SEP = LY::SEP, TA = LY::TA;
+    constexpr int BCOLS = acc_cols<NT, SPLIT, SEP>;          // one accumulator buffer
+    constexpr int ACOL = 2 * BCOLS;                          // factor ring (TA): CD x 4 KC columns
+    constexpr int TCOLS = TA ? 512 : 2 * BCOLS;
+    static_assert(ACOL + (TA ? CD * 4 * KC : 0) <= 512, "tensor memory columns");
+    unsigned char* conv = smem;                  // [CD][CONV]
+    unsigned char* raw = smem + CD * LY::CONV;   // [RD][RAW]
     uint64_t* raw_full = (uint64_t*)(smem + LY::BAR_OFF);   // [RD] loaders' copies landed (count NLOAD)
-    uint64_t* raw_empty = raw_full + RD;   // [RD] converters done reading (count NCONV)
-    uint64_t* conv_full = raw_empty + RD;  // [2] converted operands written (count NCONV)
-    uint64_t* conv_empty = conv_full + 2;  // [2] MMAs of the buffer done (tcgen05.commit)
-    uint64_t* acc_full = conv_empty + 2;   // [2] all MMAs of an item's accumulator done (tcgen05.commit)
+    uint64_t* raw_empty = raw_full + RD;   // [RD] converters done reading (count CGRP)
+    uint64_t* conv_full = raw_empty + RD;  // [CD] converted operands written (count CGRP)
+    uint64_t* conv_empty = conv_full + CD; // [CD] MMAs of the buffer done (tcgen05.commit)
+    uint64_t* acc_full = conv_empty + CD;  // [2] all MMAs of an item's accumulator done (tcgen05.commit)
     uint64_t* acc_empty = acc_full + 2;    // [2] epilogue done reading the accumulator (count NEPI)
     uint32_t* tptr = (uint32_t*)(acc_empty + 2);
     volatile int* abort = (volatile int*)tptr + 1;
@@ -497,11 +575,13 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
     if (t == 0) {
         for (int b = 0; b < RD; ++b) {
             mbar_init(raw_full + b, NLOAD);
-            mbar_init(raw_empty + b, NCONV);
+            mbar_init(raw_empty + b, CGRP);
+        }
+        for (int b = 0; b < CD; ++b) {
+            mbar_init(conv_full + b, CGRP);
+            mbar_init(conv_empty + b, 1);
         }
         for (int b = 0; b < 2; ++b) {
-            mbar_init(conv_full + b, NCONV);
-            mbar_init(conv_empty + b, 1);
             mbar_init(acc_full + b, 1);
             mbar_init(acc_empty + b, LY::NEPI);
         }
@@ -516,50 +596,62 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
 
     if (t < NLOAD) {
         // ------------------------------------------------------------ loaders
-        // the next item is decoded, and the next stage's vector rows looked up, while the
-        // current stage's copies are issued
+        // the next item is decoded, and the vector rows of the next two stages (BA: a lookup in the
+        // update list) are on their way, while the current stage's copies are issued
         long long gs = 0;  // stage counter across this block's items
         long long item = blockIdx.x;
         Item cur;
-        Vrows<NT> rows;
+        Vrows<NT> rows, rows1;
         if (item < nitems) {
             cur = decode<NT, MODE>(tasks, jobs, item, nchunks);
             rows = stage_rows<NT, MODE>(cur, 0, t);
+            rows1 = stage_rows<NT, MODE>(cur, 1, t);   // an item has at least two stages
         }
         for (; item < nitems && ok; item += gridDim.x) {
             const long long nxt_item = item + gridDim.x;
             Item nxt = cur;
             if (nxt_item < nitems) nxt = decode<NT, MODE>(tasks, jobs, nxt_item, nchunks);
+            TilePtrs<MODE> tp;
+            tp.init(cur, t);
             for (int s = 0; s < cur.nst && ok; ++s, ++gs) {
                 const int slot = (int)(gs % RD);
                 const long long use = gs / RD;
-                Vrows<NT> next_rows;
-                if (s + 1 < cur.nst) next_rows = stage_rows<NT, MODE>(cur, s + 1, t);
-                else if (nxt_item < nitems) next_rows = stage_rows<NT, MODE>(nxt, 0, t);
+                Vrows<NT> rows2;
+                if (s + 2 < cur.nst) rows2 = stage_rows<NT, MODE>(cur, s + 2, t);
+                else if (nxt_item < nitems) rows2 = stage_rows<NT, MODE>(nxt, s + 2 - cur.nst, t);
                 if (gs >= RD) ok = mbar_wait(smem_u32(raw_empty + slot), (uint32_t)((use - 1) & 1), abort, polls);
                 if (!ok) break;
-                load_stage<NT, MODE>(raw + slot * RG::RAW, cur, s, ldc, t, rows);
+                load_stage<NT, MODE>(raw + slot * RG::RAW, cur, tp, s, ldc, t, rows);
                 cp_async_arrive(raw_full + slot);
-                rows = next_rows;
+                rows = rows1;
+                rows1 = rows2;
             }
             cur = nxt;
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
     } else if (t < NLOAD + NCONV) {
         // ------------------------------------------------------------ converters
-        const int ct = t - NLOAD;
+        // two groups of warps take alternate stages: a stage is a chain of waits, shared-memory loads,
+        // operand stores and fences, and two of them overlap
+        const int ct = (t - NLOAD) & (CGRP - 1), grp = (t - NLOAD) / CGRP;
         long long gs = 0;
         int nst_next = blockIdx.x < nitems ? decode<NT, MODE>(tasks, jobs, blockIdx.x, nchunks).nst : 0;
         for (long long item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
             const int nst = nst_next;   // decoded one item ahead
             if (item + gridDim.x < nitems) nst_next = decode<NT, MODE>(tasks, jobs, item + gridDim.x, nchunks).nst;
             for (int s = 0; s < nst && ok; ++s, ++gs) {
-                const int slot = (int)(gs % RD), cb = (int)(gs & 1);
-                const long long use = gs / RD, cuse = gs >> 1;
+                if ((int)(gs & 1) != grp) continue;
+                const int slot = (int)(gs % RD), cb = (int)(gs % CD);
+                const long long use = gs / RD, cuse = gs / CD;
                 ok = mbar_wait(smem_u32(raw_full + slot), (uint32_t)(use & 1), abort, polls);
-                if (ok && gs >= 2) ok = mbar_wait(smem_u32(conv_empty + cb), (uint32_t)((cuse - 1) & 1), abort, polls);
-                if (!ok) break;
-                convert_stage<NT, MODE, SPLIT>(raw + slot * RG::RAW, conv + cb * RG::CONV, ct);
+                if (ok && gs >= CD) ok = mbar_wait(smem_u32(conv_empty + cb), (uint32_t)((cuse - 1) & 1), abort, polls);
+                if (!TA && !ok) break;
+                if (TA) {
+                    ok = __all_sync(0xffffffffu, ok);   // the tensor-memory stores are warp-wide
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                }
+                convert_stage<NT, MODE, SPLIT, TA, CGRP>(raw + slot * RG::RAW, conv + cb * LY::CONV, ct, tmem + ACOL + cb * 4 * KC);
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 mbar_arrive(raw_empty + slot);
                 mbar_arrive(conv_full + cb);
@@ -580,11 +672,11 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t tm = tmem + (uint32_t)(b * BCOLS);
                 for (int s = 0; s < nst && ok; ++s, ++gs) {
-                    const int cb = (int)(gs & 1);
-                    ok = mbar_wait(smem_u32(conv_full + cb), (uint32_t)((gs >> 1) & 1), abort, polls);
+                    const int cb = (int)(gs % CD);
+                    ok = mbar_wait(smem_u32(conv_full + cb), (uint32_t)((gs / CD) & 1), abort, polls);
                     if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    mma_item_stage<NT, SPLIT, SEP>(smem_u32(conv + cb * RG::CONV), tm, s == 0);
+                    mma_item_stage<NT, SPLIT, SEP, TA>(smem_u32(conv + cb * LY::CONV), tm, s == 0, tmem + ACOL + cb * 4 * KC);
                     mma_commit(conv_empty + cb);
                 }
                 mma_commit(acc_full + b);   // arrives when every MMA issued so far has completed

@@ -38,10 +38,9 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
 // byte offset of (row, k) in a [rows x KC] K-major core-matrix operand (4-byte elements)
 __device__ __forceinline__ int coff(int row, int k) { return (row >> 3) * SBO + (k >> 2) * LBO + (row & 7) * 16 + (k & 3) * 4; }
 
+// v rounded to TF32 (10 mantissa bits), to nearest with ties away from zero, in two integer operations
 __device__ __forceinline__ float tf32_hi(float v) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(v));
-    return __uint_as_float(r);
+    return __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xffffe000u);
 }
 
 // 16-byte asynchronous global->shared copy; src_bytes = 0 zero-fills without reading
@@ -81,6 +80,19 @@ __device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uin
     asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
                  "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}"
                  :: "r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc));
+}
+
+// the same with the A operand in tensor memory
+__device__ __forceinline__ void mma_tf32_ta(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                 "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}"
+                 :: "r"(d), "r"(a), "l"(b), "r"(idesc), "r"(acc));
+}
+
+// 8 columns of this warp's 32 tensor-memory lanes
+__device__ __forceinline__ void tmem_st8(uint32_t a, const float (&v)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 :: "r"(a), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]));
 }
 
 __device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
@@ -152,27 +164,32 @@ __device__ __forceinline__ void mma_stage(uint32_t base, uint32_t tm_r, uint32_t
 // a real factor part's products with both vector parts, so the factor operand is read from shared
 // memory 6 times per 8 indices instead of 12, and NT = 64 runs at the N = 128 rate.  The vector
 // operand holds [-Xi | Xr | Xi] (3 NT rows) for hi, then for lo; [Yr | Yi] += Ar [Xr | Xi] +
-// Ai [-Xi | Xr], hi x hi terms at tm, the others (SPLIT = 3) at tm + 2 NT.
-template <int NT, int SPLIT>
-__device__ __forceinline__ void mma_stage_wide(uint32_t base, uint32_t tm, bool first_stage) {
+// Ai [-Xi | Xr], hi x hi terms at tm, the others (SPLIT = 3) at tm + 2 NT (SEP) or with them.
+// TA: the factor operand is in tensor memory (16 columns each of Ar_hi, Ar_lo, Ai_hi, Ai_lo from column
+// ta on, lane = row), and `base` holds the vector operand alone.
+template <int NT, int SPLIT, bool SEP, bool TA>
+__device__ __forceinline__ void mma_stage_wide(uint32_t base, uint32_t tm, bool first_stage, uint32_t ta) {
     constexpr int A_MAT = MR * KC * 4, X_MAT = NT * KC * 4;
+    const uint32_t tl = SEP ? tm + 2 * NT : tm;
     const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(2 * NT >> 3) << 17) | ((uint32_t)(MR >> 4) << 24);
 #pragma unroll
     for (int ks = 0; ks < KC / 8; ++ks) {
         const uint32_t ko = ks * 2 * LBO;
-        const uint64_t arh = smem_desc(base + 0 * A_MAT + ko), arl = smem_desc(base + 1 * A_MAT + ko);
-        const uint64_t aih = smem_desc(base + 2 * A_MAT + ko), ail = smem_desc(base + 3 * A_MAT + ko);
-        const uint32_t xb = base + 4 * A_MAT + ko;
+        auto mma = [&](uint32_t d, int mat, uint64_t x, uint32_t acc) {   // mat: 0 Ar_hi, 1 Ar_lo, 2 Ai_hi, 3 Ai_lo
+            if constexpr (TA) mma_tf32_ta(d, ta + mat * KC + ks * 8, x, idesc, acc);
+            else mma_tf32(d, smem_desc(base + mat * A_MAT + ko), x, idesc, acc);
+        };
+        const uint32_t xb = base + (TA ? 0 : 4 * A_MAT) + ko;
         const uint64_t nrh = smem_desc(xb), rih = smem_desc(xb + X_MAT);   // [-Xi | Xr], [Xr | Xi]
         const uint32_t first = (first_stage && ks == 0) ? 0u : 1u;
-        mma_tf32(tm, arh, rih, idesc, first);
-        mma_tf32(tm, aih, nrh, idesc, 1u);
+        mma(tm, 0, rih, first);
+        mma(tm, 2, nrh, 1u);
         if (SPLIT == 3) {
             const uint64_t nrl = smem_desc(xb + 3 * X_MAT), ril = smem_desc(xb + 4 * X_MAT);
-            mma_tf32(tm + 2 * NT, arh, ril, idesc, first);
-            mma_tf32(tm + 2 * NT, arl, rih, idesc, 1u);
-            mma_tf32(tm + 2 * NT, aih, nrl, idesc, 1u);
-            mma_tf32(tm + 2 * NT, ail, nrh, idesc, 1u);
+            mma(tl, 0, ril, SEP ? first : 1u);
+            mma(tl, 1, rih, 1u);
+            mma(tl, 2, nrl, 1u);
+            mma(tl, 3, nrh, 1u);
         }
     }
 }
