@@ -99,67 +99,119 @@ __global__ void k_extend_add(const ExtDesc<C>* ed) {
     }
 }
 
-// Diagonal block of panel k0: unpivoted LDL^T in FP64 in shared memory, D and D^{-1}
-// stored, and the inverse of the unit lower block written as the packed diagonal tile.
+// Diagonal block of panel k0: unpivoted LDL^T in FP64, D and D^{-1} stored, and the inverse of the
+// unit lower block written as the packed diagonal tile.
+//
+// Bound by the FP64 pipe (2 lanes per clock and SM) and by the chain of 32 pivots.  The block lives in
+// registers: warp w holds columns w, w + 8, w + 16, w + 24, lane = row.  Eliminating column k subtracts
+// l_ik times row k from the rows below in both halves of [A | I] at once: an entry is A_ij until its
+// column is eliminated (then L_ij is written out) and X_ij = (L^{-1})_ij from there on, so every step is
+// four fused multiply-adds per entry and one block barrier, with the next pivot's reciprocal formed
+// ahead of the other columns' updates.  From row 16 on the upper half of the rows is final, and
+// the lower half's four columns are spread over all 32 lanes.  (Updates of the whole square in shared memory
+// and a substitution by one warp for the inverse took 223 us a launch at 64^3, 8 layers; this takes 104,
+// most of it the pivots' dependent FP64 operations queued behind the other columns' updates.)
+__device__ __forceinline__ double2 shfl2(double2 v, int src) {
+    return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+__device__ __forceinline__ void msub(double2& v, double2 l, double2 m) {   // v -= l m
+    v.x = fma(-l.x, m.x, v.x); v.x = fma(l.y, m.y, v.x);
+    v.y = fma(-l.x, m.y, v.y); v.y = fma(-l.y, m.x, v.y);
+}
+
 template <class C>
-__global__ void k_diag(const FrontDesc<C>* fd, int k0, int* flag) {
+__global__ void __launch_bounds__(256) k_diag(const FrontDesc<C>* fd, int k0, int* flag) {
     const FrontDesc<C>& f = fd[blockIdx.x];
     if (k0 >= f.nown) return;
     const int nb = min(TILE, f.nown - k0);
-    __shared__ double2 a[TILE][TILE + 1];
-    __shared__ double2 xinv[TILE][TILE + 1];
-    __shared__ double2 dinv_s[TILE];
-    const int t = threadIdx.x;
-    for (int q = t; q < TILE * TILE; q += blockDim.x) {
-        int i = q % TILE, j = q / TILE;
-        double2 v = make_double2(0.0, 0.0);
-        if (i < nb && j < nb && i >= j) v = to_d(f.F[(long long)(k0 + i) + (long long)(k0 + j) * f.m]);
-        a[i][j] = v;
+    __shared__ double2 us[2][TILE], ls[2][TILE];   // column k before and after scaling, by parity of k
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    C* F = f.F + (long long)k0 * (f.m + 1);        // (row, col) of the block at row + col * m
+    C* tile = f.fac + (f.linv_off + tri_index(k0 / TILE, k0 / TILE)) * TILE2;
+    double2 v[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const int j = w + 8 * c;
+        v[c] = (lane < nb && j <= lane) ? to_d(F[(long long)lane + (long long)j * f.m]) : make_double2(0.0, 0.0);
     }
-    __syncthreads();
-    for (int k = 0; k < nb; ++k) {
-        double2 d = a[k][k];
-        double dd = d.x * d.x + d.y * d.y;
-        if (t == 0) {
-            if (!(dd > 1e-280) || !isfinite(dd)) atomicExch(flag, 1);
-            dinv_s[k] = (dd > 0.0) ? crecip(d) : make_double2(0.0, 0.0);
-        }
-        __syncthreads();
-        double2 di = dinv_s[k];
-        int cnt = nb - k - 1;
-        for (int q = t; q < cnt * cnt; q += blockDim.x) {
-            int i = k + 1 + q % cnt, j = k + 1 + q / cnt;
-            if (i >= j) a[i][j] = csub(a[i][j], cmul(cmul(a[i][k], di), a[j][k]));
-        }
-        __syncthreads();
-        for (int i = k + 1 + t; i < nb; i += blockDim.x) a[i][k] = cmul(a[i][k], di);
-        __syncthreads();
-    }
-    // inverse of the unit lower triangular block, one column per thread
-    if (t < TILE) {
-        int j = t;
-        for (int i = 0; i < TILE; ++i) xinv[i][j] = make_double2(0.0, 0.0);
-        if (j < nb) {
-            xinv[j][j] = make_double2(1.0, 0.0);
-            for (int i = j + 1; i < nb; ++i) {
-                double2 s = make_double2(0.0, 0.0);
-                for (int k = j; k < i; ++k) s = cadd(s, cmul(a[i][k], xinv[k][j]));
-                xinv[i][j] = cneg(s);
+    // column k by its owner warp, whose lanes `row` >= k hold it in x: pivot, L, D^{-1}; x becomes X's column
+    auto pivot = [&](double2& x, int k, int row, bool holds) {
+        const double2 d = shfl2(x, k);             // row k sits in lane k in both layouts
+        const double dd = d.x * d.x + d.y * d.y;
+        const double2 di = (dd > 0.0) ? crecip(d) : make_double2(0.0, 0.0);
+        const double2 l = (holds && row > k) ? cmul(x, di) : make_double2(0.0, 0.0);
+        if (holds) {
+            us[k & 1][row] = x;
+            ls[k & 1][row] = l;
+            if (row >= k && row < nb) F[(long long)row + (long long)k * f.m] = from_d<C>(row == k ? d : l);
+            if (row == k) {
+                if (!(dd > 1e-280) || !isfinite(dd)) atomicExch(flag, 1);
+                f.dinv[f.own0 + k0 + k] = from_d<C>(di);
             }
+            x = make_double2(row == k ? 1.0 : 0.0, 0.0);
+        }
+    };
+    // rows 0 .. 31 in lanes, four columns each
+    if (w == 0) pivot(v[0], 0, lane, true);
+    __syncthreads();
+    const int n1 = min(nb, 16);
+    for (int k = 0; k < n1; ++k) {
+        const double2 l = ls[k & 1][lane];
+        const int kn = k + 1;                       // next pivot: its column first, then its reciprocal
+        const bool own = kn < nb && kn < 16 && w == (kn & 7);
+        auto update = [&](int c) {
+            const int j = w + 8 * c;
+            const double2 m = j > k ? us[k & 1][j] : shfl2(v[c], k);
+            msub(v[c], l, m);
+        };
+        if (own) {
+            if (kn < 8) { update(0); pivot(v[0], kn, lane, true); }
+            else { update(1); pivot(v[1], kn, lane, true); }
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (!(own && c == (kn >> 3))) update(c);
+        __syncthreads();
+    }
+    // rows 0 .. 15 of the inverse are final
+    if (lane < 16) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tile[lane + (w + 8 * c) * TILE] = from_d<C>(w + 8 * c <= lane ? v[c] : make_double2(0.0, 0.0));
+    }
+    // rows 16 .. 31: lanes 0 .. 15 take columns w, w + 8, lanes 16 .. 31 columns w + 16, w + 24
+    const int row = 16 + (lane & 15), jh = w + (lane & 16);
+    double2 y[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const double2 lo = shfl2(v[c], row);
+        y[c] = lane < 16 ? lo : v[c + 2];
+    }
+    if (nb > 16) {
+        if (w == 0) pivot(y[0], 16, row, lane >= 16);
+        __syncthreads();
+        for (int k = 16; k < nb; ++k) {
+            const double2 l = ls[k & 1][row];
+            const int kn = k + 1;
+            const bool own = kn < nb && w == (kn & 7);
+            auto update = [&](int c) {
+                const int j = jh + 8 * c;
+                const double2 x = shfl2(y[c], (lane & 16) | (k & 15));
+                msub(y[c], l, j > k ? us[k & 1][j] : x);
+            };
+            if (own) {
+                if (kn < 24) { update(0); pivot(y[0], kn, row, lane >= 16); }
+                else { update(1); pivot(y[1], kn, row, lane >= 16); }
+            }
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+                if (!(own && c == ((kn >> 3) & 1))) update(c);
+            __syncthreads();
         }
     }
-    __syncthreads();
-    // write back: strict lower L, D on the diagonal, D^{-1}, packed inverse tile
-    for (int q = t; q < nb * nb; q += blockDim.x) {
-        int i = q % nb, j = q / nb;
-        if (i >= j) f.F[(long long)(k0 + i) + (long long)(k0 + j) * f.m] = from_d<C>(a[i][j]);
-    }
-    for (int k = t; k < nb; k += blockDim.x) f.dinv[f.own0 + k0 + k] = from_d<C>(dinv_s[k]);
-    const int kt = k0 / TILE;
-    C* tile = f.fac + (f.linv_off + tri_index(kt, kt)) * TILE2;
-    for (int q = t; q < TILE2; q += blockDim.x) {
-        int i = q % TILE, j = q / TILE;
-        tile[q] = from_d<C>(xinv[i][j]);
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const int j = jh + 8 * c;
+        tile[row + j * TILE] = from_d<C>(j <= row ? y[c] : make_double2(0.0, 0.0));
     }
 }
 
