@@ -528,8 +528,12 @@ template <int NT> struct PLayout {
     static constexpr bool TA = RG::WIDE;
     // the hi x lo terms' own accumulators fit beside the factor ring at NT = 32
     static constexpr bool SEP = NT == 32;
-    static constexpr int CD = NT == 32 ? 4 : NT == 64 ? 3 : 2;     // converted operands' ring depth
+    static constexpr int CD = NT <= 64 ? 4 : 2;                    // converted operands' ring depth
     static constexpr int RD = NT == 32 ? 6 : NT == 64 ? 4 : 2;     // raw ring depth
+    // A converter group must have filled a ring slot's previous stage itself: a parity wait tells only
+    // the last phase from the one before, so it may not be reached while an older use is still open.
+    // Two groups take alternate stages, so both depths are even.
+    static_assert(CD % 2 == 0 && RD % 2 == 0, "a ring slot belongs to one converter group");
     static constexpr int CONV = TA ? 6 * RG::X_MAT : RG::CONV;
     static constexpr int NEPI = 128;                       // epilogue threads (4 warps)
     static constexpr int NTHREADS = NLOAD + NCONV + 32 + NEPI;
@@ -537,6 +541,7 @@ template <int NT> struct PLayout {
     static constexpr int STG_OFF = CD * CONV + RD * RG::RAW;   // 4 warps x 32 rows x EP complex
     static constexpr int BAR_OFF = STG_OFF + 4 * 32 * EP * 8;
     static constexpr int TOTAL = BAR_OFF + (2 * RD + 2 * CD + 4) * 8 + 16;
+    static_assert(TOTAL <= 232448, "shared memory of one block");
 };
 
 template <int NT, int MODE, int SPLIT>
