@@ -955,10 +955,20 @@ void rec_volume_sources(Ctx& ctx, Rec& rec, const std::vector<int>& layers, cons
     });
 }
 
+// A bounded wait that gave up in a substitution (every width has such waits) is an error here too.
+inline void check_waits(Ctx& ctx) {
+    int flag = 0;
+    HZ_CUDA(cudaMemcpyAsync(&flag, ctx.d_flag + 1, sizeof(int), cudaMemcpyDeviceToHost, ctx.stream));
+    HZ_CUDA(cudaStreamSynchronize(ctx.stream));
+    if (!flag) return;
+    HZ_CUDA(cudaMemsetAsync(ctx.d_flag + 1, 0, sizeof(int), ctx.stream));
+    throw Error{HZ_ERR_TIMEOUT, "a substitution block gave up on one of its waits"};
+}
+
 // run a freshly recorded operator once and release its descriptors
 inline void run_now(Ctx& ctx, Rec& rec) {
     rec.run(ctx.stream);
-    HZ_CUDA(cudaStreamSynchronize(ctx.stream));
+    check_waits(ctx);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1229,7 +1239,7 @@ void build_trace_blocks(Ctx& ctx, int chunk) {
             k_store_blocks<C><<<g2, 256, 0, ctx.stream>>>((C*)tb.base, d_off, T, n2, chunk, k0);
             HZ_CHECK_LAUNCH();
         }
-        HZ_CUDA(cudaStreamSynchronize(ctx.stream));
+        check_waits(ctx);
     } catch (...) {
         cudaStreamSynchronize(ctx.stream);
         cleanup();
