@@ -217,6 +217,7 @@ __device__ __forceinline__ bool run_task(const STask& tk, const JobDev<float2>& 
         asm volatile("cp.async.wait_group %0;" :: "n"(DX - 1) : "memory");
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
+        __syncwarp();   // the slice holds pieces that other lanes copied: a vote orders no memory accesses
         ++u;
         const float2* tile = (const float2*)(ts.ring + slot * SLOT);
         const float2* x = (const float2*)(xs + (j % DX) * LY::XS);

@@ -1,0 +1,53 @@
+"""The one-launch substitution (complex64 blocks of at most 16 columns) against the complex128 local
+solves, one launch per substitution, at tolerances near its own error.
+
+Tolerances: a local solve on complex64 factors is 1e-5 to 3e-5 off at 40^3 to 56^3 cells a layer, so 4e-5
+on the boxes here (at most 20 000 cells); on rounded complex128 factors the products' FP32 rounding is
+left, some 30 roundings of 6e-8 along a chain of products: 5e-6."""
+import numpy as np
+import pytest
+
+from paper_1801_08655_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL = {"mixed": 4e-5, "mixed64": 5e-6}
+
+
+def one_layer(shape, precision, stream=None, seed=0):
+    from paper_1801_08655_gb300 import hz
+    rng = np.random.default_rng(seed + sum(shape))
+    c = 1.5 + rng.random(shape)
+    s = hz.Solver(1.0 / (c * c), W.omega_for_ppw(1.5, 9.0), 1, W.pml_constant(2.5), 1, precision=precision,
+                  stream=stream)
+    s.factor()
+    return s
+
+
+def sources(shape, R, seed):
+    g = torch.Generator("cuda").manual_seed(seed)
+    return torch.randn((R,) + shape, dtype=torch.complex128, device="cuda", generator=g)
+
+
+def rel(a, b):
+    return float((a - b).norm() / b.norm())
+
+
+@pytest.mark.parametrize("precision", ["mixed", "mixed64"])
+@pytest.mark.parametrize("shape", [(9, 33, 10), (21, 24, 23), (24, 28, 30)])
+def test_every_width_in_one_launch(shape, precision):
+    from paper_1801_08655_gb300 import build
+    build.build()
+    s, ref = one_layer(shape, precision), one_layer(shape, "fp64")
+    for R in range(1, 17):
+        g = sources(shape, R, R)
+        want = ref.layer_solve(0, g)
+        s.layer_solve(0, g)
+        s.profile_begin(detail=True)
+        got = s.layer_solve(0, g)
+        s.profile_end()
+        assert s.profile_kernel(0)["launches"] == 1 and s.profile_kernel(1)["launches"] == 0, R
+        assert rel(got, want) < TOL[precision], (R, rel(got, want))
+    s.close()
+    ref.close()
