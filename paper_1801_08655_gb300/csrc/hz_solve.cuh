@@ -13,6 +13,30 @@ int padded_ldc(bool is_double, int ncols);
 // one-launch substitution of complex64 blocks (subst_stream.cu): usable for this leading dimension;
 // task lists of a batch's active products; the launch (sync: two counters, zero between launches)
 bool stream_usable(int ldc);
+// One task, as the host lays it out: the tile of step j sits at tile0 + j step + dstep j (j - 1) / 2.
+struct STask {
+    long long tile0;
+    long long upd_off;    // of the node's update indices
+    int mode, job;
+    int nunits, half0;    // steps of SKU reduction indices; whether the first is a tile's second half
+    int step, dstep;
+    int own0;             // first own row of the node
+    int k0, nk;           // first reduction row of the range (own or update position), rows from there on
+    int row0, nrows;      // first output row (own or update position), rows of this slab (<= TILE)
+    int store;            // 1: the task is its rows' only writer
+};
+static_assert(sizeof(STask) == 64, "one 64-byte load per task");
+constexpr int SKU = 16;                      // reduction indices per step (half a tile)
+enum { ST_ZERO_ACC = 4, ST_ZERO_X = 5 };     // modes besides the products': clear the rows of a split FA / BB output
+// Tasks of `warps` warps, each one's phases in order, with off[warp * nph + phase] the first task of
+// each; one task more than off.back() at the end (read ahead, never run).  Host only.
+struct StreamLists {
+    std::vector<STask> tasks;
+    std::vector<int> off;
+    int nph = 0;
+};
+StreamLists stream_lists(const Ctx& ctx, const std::vector<int>& layers, const std::vector<StreamProduct>& prods, int H,
+                         int warps);
 void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vector<StreamProduct>& prods, int H,
                   StreamPlan& plan);
 void launch_stream(const StreamPlan& p, const void* jobs, int ldc, unsigned* sync, int* flag, long long polls,
@@ -39,6 +63,23 @@ inline int blocked_code(int nblk, const int* codes) {
 }
 inline int block_count(int sparse) { return (sparse & SP_BLOCKS) ? (sparse >> 17) & 7 : 1; }
 inline int block_code(int sparse, int q) { return (sparse & SP_BLOCKS) ? (sparse >> (4 * q)) & 15 : sparse; }
+
+// Task lists of a batch: CUDA-core tasks and tensor-core items by phase (FA, FB, BA, BB) and level, the
+// active products of the one-launch form instead of either, the own rows to clear before the phase that
+// adds into them, and the algorithmic work per [tensor cores][phase][level].  Host only: no device
+// memory is read or allocated.  elem: bytes of a factor entry (8: complex64, on M21; 16: complex128, on L21).
+struct ZeroRows { int layer; bool x; int own0, nown; };   // layer: position in the batch; x or acc
+struct BatchLists {
+    int H = 0;
+    std::vector<std::vector<Task>> lists[4], quads[4];
+    std::vector<StreamProduct> prods;
+    std::vector<ZeroRows> zero;
+    std::vector<double> bytes[2][4], flops[2][4];
+};
+BatchLists batch_lists(const Ctx& ctx, const std::vector<int>& layers, size_t elem, int KS, bool tc, int KS_tc, int min_t,
+                       int sparse, bool stream);
+// Candidates that the tuner times for this leading dimension.  Host only.
+std::vector<Ctx::TuneChoice> tune_candidates(const Ctx& ctx, bool is_double, int ncols);
 
 // Job set with per-level task lists, cached by layer list and sparsity code.
 template <class C> Batch& get_batch(Ctx& ctx, const std::vector<int>& layers, int ncols, int split = 3, int sparse = 0);

@@ -555,14 +555,9 @@ Batch& get_batch(Ctx& ctx, const std::vector<int>& layers, int ncols, int split,
     return get_batch_cfg<C>(ctx, layers, ncols, KS, 0, tc, KS_tc, ctx.tc_min_tiles, split, ctx.tc_cfg, sparse);
 }
 
-template <class C>
-void ensure_tuned(Ctx& ctx, const std::vector<int>& layers, int ncols, int split, int sparse) {
-    const bool dbl = sizeof(C) == 16;
+std::vector<Ctx::TuneChoice> tune_candidates(const Ctx& ctx, bool dbl, int ncols) {
     const int ldc = padded_ldc(dbl, ncols);
     const bool tc_ok = !dbl && tc_usable(ctx, ldc);
-    const std::string key = tune_key(ctx, layers, ldc, split, sparse);
-    if (!ctx.autotune || ctx.tuned.count(key)) return;
-    if (!dbl && use_one_launch(ctx, ldc, sparse)) return;   // get_batch takes it without timing
     const int cc0 = chunk_cols(dbl, ncols);
     std::vector<Ctx::TuneChoice> cands;
     const bool try_tc = tc_ok && ctx.tc_mode >= 1;
@@ -588,6 +583,17 @@ void ensure_tuned(Ctx& ctx, const std::vector<int>& layers, int ncols, int split
             for (int kstc : {4, 1 << 30}) cands.push_back({8, cc0, 1, kstc, mt, 0});
         }
     }
+    return cands;
+}
+
+template <class C>
+void ensure_tuned(Ctx& ctx, const std::vector<int>& layers, int ncols, int split, int sparse) {
+    const bool dbl = sizeof(C) == 16;
+    const int ldc = padded_ldc(dbl, ncols);
+    const std::string key = tune_key(ctx, layers, ldc, split, sparse);
+    if (!ctx.autotune || ctx.tuned.count(key)) return;
+    if (!dbl && use_one_launch(ctx, ldc, sparse)) return;   // get_batch takes it without timing
+    const std::vector<Ctx::TuneChoice> cands = tune_candidates(ctx, dbl, ncols);
     cudaEvent_t e0, e1;
     HZ_CUDA(cudaEventCreate(&e0));
     HZ_CUDA(cudaEventCreate(&e1));
@@ -622,48 +628,21 @@ void ensure_tuned(Ctx& ctx, const std::vector<int>& layers, int ncols, int split
     ctx.tune_log.push_back(log);
 }
 
-template <class C>
-Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS, int CC, bool tc, int KS_tc,
-                     int min_t, int split, int tc_cfg, int sparse, bool stream) {
-    const bool dbl = sizeof(C) == 16;
-    const int ldc = padded_ldc(dbl, ncols);
-    std::string key = "KS" + std::to_string(KS) + "C" + std::to_string(CC) + "n" + std::to_string(ldc) +
-                      (tc ? "tc" + std::to_string(KS_tc) + "m" + std::to_string(min_t) + "s" + std::to_string(split) +
-                                "c" + std::to_string(tc_cfg)
-                          : stream ? "st" : "") + "p" + std::to_string(sparse) + ":";
-    for (int l : layers) key += std::to_string(l) + ",";
-    auto it = ctx.batches.find(key);
-    if (it != ctx.batches.end()) return it->second;
-    Batch b;
-    b.layers = layers;
-    b.KS = KS;
-    b.CC = CC;
-    b.tc = tc;
-    b.KS_tc = KS_tc;
-    b.min_t = min_t;
-    b.split = split;
-    b.tc_cfg = tc_cfg;
-    b.sparse = sparse;
-    b.wait_polls = ctx.tc_wait_polls;
-    b.stream = stream;
-    std::vector<StreamProduct> prods;
-    // per-block sparsity: job j * nblk + q is block q (columns [q * job_cols, (q + 1) * job_cols))
-    // of layer j; the caller has checked that the blocks tile the columns in whole chunks
+BatchLists batch_lists(const Ctx& ctx, const std::vector<int>& layers, size_t elem, int KS, bool tc, int KS_tc, int min_t,
+                       int sparse, bool stream) {
+    BatchLists out;
+    const bool m21 = elem == sizeof(float2);
     const int nblk = block_count(sparse);
-    if (nblk > 1 && (ncols % nblk != 0 || (ncols / nblk) % 64 != 0 || ldc != ncols))
-        throw Error{HZ_ERR_ARG, "per-block sparsity needs column blocks of a multiple of 64"};
-    b.job_cols = nblk > 1 ? ncols / nblk : 0;
     int H = 0;
     for (int l : layers) H = std::max(H, (int)ctx.shapes[ctx.layers[l].shape].levels.size());
-    b.H = H;
-    const bool m21 = has_m21<C>;
-    std::vector<std::vector<Task>> lists[4], quads[4];
+    out.H = H;
+    auto &lists = out.lists, &quads = out.quads;
     for (auto& v : lists) v.assign(H, {});
     for (auto& v : quads) v.assign(H, {});
     for (int k = 0; k < 2; ++k)
         for (int mode = 0; mode < 4; ++mode) {
-            b.lvl_bytes[k][mode].assign(H, 0.0);
-            b.lvl_flops[k][mode].assign(H, 0.0);
+            out.bytes[k][mode].assign(H, 0.0);
+            out.flops[k][mode].assign(H, 0.0);
         }
     auto add_tasks = [&](std::vector<Task>& out, int j, int nid, int tile, int k0, int k1, int ks) {
         if (k1 >= 65536) throw Error{HZ_ERR_ARG, "node product too long"};
@@ -677,7 +656,6 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
     auto diag_ks = [&](const Node& nd, int ks) {
         return std::min(std::max(ks, 16), nd.parent < 0 ? std::max(1, (nd.own_t + 1) / 2) : 1 << 30);
     };
-    std::vector<ZeroDev> zero_rows[2];   // acc, x
     for (int j = 0; j < (int)layers.size(); ++j) {
         const Layer& ly = ctx.layers[layers[j]];
         const Shape& sh = ctx.shapes[ly.shape];
@@ -713,9 +691,9 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
                 for (int mode = 0; mode < 4; ++mode) {
                     const bool fwd = mode == FA || mode == FB;
                     const int out_t = mode == 1 ? nd.upd_t : nd.own_t;
-                    const bool on_tc = tc && tc_node(mode, nd, b.min_t);
+                    const bool on_tc = tc && tc_node(mode, nd, min_t);
                     const bool diag = m21 && (mode == 0 || mode == 3);
-                    const int ks_tc = diag ? diag_ks(nd, b.KS_tc) : b.KS_tc, ks = diag ? diag_ks(nd, KS) : KS;
+                    const int ks_tc = diag ? diag_ks(nd, KS_tc) : KS_tc, ks = diag ? diag_ks(nd, KS) : KS;
                     int nact = 0;
                     if (m21 && mode == 2 && nd.nupd == 0) continue;   // the root has nothing to gather
                     // M21: FA and BB of every level go in one launch each
@@ -730,7 +708,7 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
                         ++nact;
                         const int jq = j * nblk + q;
                         if (stream) {
-                            prods.push_back({mode, h, jq, nid});
+                            out.prods.push_back({mode, h, jq, nid});
                         } else if (on_tc) {
                             for (int t = 0; t < out_t; t += 4) {
                                 if (mode == 0) add_tasks(quads[0][hl], jq, nid, t, 0, std::min(t + 4, nd.own_t), ks_tc);
@@ -748,16 +726,13 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
                         }
                     }
                     if (nact == 0) continue;
-                    if (diag && nd.own_t > (on_tc ? ks_tc : ks)) {
-                        C* v = (C*)(mode == 0 ? ctx.slot_x[layers[j]] : ctx.slot_acc[layers[j]]) + (long long)nd.own0 * ldc;
-                        zero_rows[mode == 0].push_back({v, (long long)nd.nown * ldc * (long long)sizeof(C)});
-                    }
+                    if (diag && nd.own_t > (on_tc ? ks_tc : ks)) out.zero.push_back({j, mode == 0, nd.own0, nd.nown});
                     // stored factor entries this product reads (triangular L^{-1} or L21): once
                     // algorithmically, however many column blocks use them
                     const double ent = (mode == FA || mode == BB) ? (double)nd.nown * (nd.nown + 1) / 2.0
                                                                   : (double)nd.nown * nd.nupd;
-                    b.lvl_bytes[on_tc][mode][hl] += ent * sizeof(C);
-                    b.lvl_flops[on_tc][mode][hl] += 8.0 * ent * nact / nblk;
+                    out.bytes[on_tc][mode][hl] += ent * (double)elem;
+                    out.flops[on_tc][mode][hl] += 8.0 * ent * nact / nblk;
                 }
             }
     }
@@ -771,6 +746,53 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
             sort_items(quads[mode][h]);
             if (m21) sort_items(lists[mode][h]);
         }
+    return out;
+}
+
+template <class C>
+Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS, int CC, bool tc, int KS_tc,
+                     int min_t, int split, int tc_cfg, int sparse, bool stream) {
+    const bool dbl = sizeof(C) == 16;
+    const int ldc = padded_ldc(dbl, ncols);
+    std::string key = "KS" + std::to_string(KS) + "C" + std::to_string(CC) + "n" + std::to_string(ldc) +
+                      (tc ? "tc" + std::to_string(KS_tc) + "m" + std::to_string(min_t) + "s" + std::to_string(split) +
+                                "c" + std::to_string(tc_cfg)
+                          : stream ? "st" : "") + "p" + std::to_string(sparse) + ":";
+    for (int l : layers) key += std::to_string(l) + ",";
+    auto it = ctx.batches.find(key);
+    if (it != ctx.batches.end()) return it->second;
+    Batch b;
+    b.layers = layers;
+    b.KS = KS;
+    b.CC = CC;
+    b.tc = tc;
+    b.KS_tc = KS_tc;
+    b.min_t = min_t;
+    b.split = split;
+    b.tc_cfg = tc_cfg;
+    b.sparse = sparse;
+    b.wait_polls = ctx.tc_wait_polls;
+    b.stream = stream;
+    // per-block sparsity: job j * nblk + q is block q (columns [q * job_cols, (q + 1) * job_cols))
+    // of layer j; the caller has checked that the blocks tile the columns in whole chunks
+    const int nblk = block_count(sparse);
+    if (nblk > 1 && (ncols % nblk != 0 || (ncols / nblk) % 64 != 0 || ldc != ncols))
+        throw Error{HZ_ERR_ARG, "per-block sparsity needs column blocks of a multiple of 64"};
+    b.job_cols = nblk > 1 ? ncols / nblk : 0;
+    const bool m21 = has_m21<C>;
+    BatchLists ls = batch_lists(ctx, layers, sizeof(C), KS, tc, KS_tc, min_t, sparse, stream);
+    const int H = b.H = ls.H;
+    auto &lists = ls.lists, &quads = ls.quads;
+    for (int k = 0; k < 2; ++k)
+        for (int mode = 0; mode < 4; ++mode) {
+            b.lvl_bytes[k][mode] = ls.bytes[k][mode];
+            b.lvl_flops[k][mode] = ls.flops[k][mode];
+        }
+    std::vector<ZeroDev> zero_rows[2];   // acc, x
+    for (const ZeroRows& z : ls.zero) {
+        void* v = z.x ? ctx.slot_x[layers[z.layer]] : ctx.slot_acc[layers[z.layer]];
+        zero_rows[z.x].push_back({(C*)v + (long long)z.own0 * ldc, (long long)z.nown * ldc * (long long)sizeof(C)});
+    }
     std::vector<Task> all;
     for (int mode = 0; mode < 4; ++mode) {
         b.pair_off[mode].assign(H, 0);
@@ -818,7 +840,7 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
                 b.alg_bytes += b.lvl_bytes[k][mode][h];
                 b.flops_per_col += b.lvl_flops[k][mode][h];
             }
-    if (stream) build_stream(ctx, layers, prods, H, b.plan);
+    if (stream) build_stream(ctx, layers, ls.prods, H, b.plan);
     for (int w = 0; w < 2; ++w) {
         std::vector<ZeroDev>& zd = zero_rows[w];
         if (!m21)

@@ -49,23 +49,8 @@ using tcc::smem_u32;
 
 enum { FA = 0, FB = 1, BA = 2, BB = 3 };
 
-// One task, as the host lays it out: the tile of step j sits at tile0 + j step + dstep j (j - 1) / 2.
-struct STask {
-    long long tile0;
-    long long upd_off;    // of the node's update indices
-    int mode, job;
-    int nunits, half0;    // steps of KU reduction indices; whether the first is a tile's second half
-    int step, dstep;
-    int own0;             // first own row of the node
-    int k0, nk;           // first reduction row of the range (own or update position), rows from there on
-    int row0, nrows;      // first output row (own or update position), rows of this slab (<= TILE)
-    int store;            // 1: the task is its rows' only writer
-};
-static_assert(sizeof(STask) == 64, "one 64-byte load per task");
-constexpr int ZERO_ACC = 4, ZERO_X = 5;   // modes: clear the rows of a split FA / BB output
-
 constexpr int SW = 8;                     // warps
-constexpr int KU = 16;                    // reduction indices per step
+constexpr int KU = SKU;                   // reduction indices per step
 constexpr int TPITCH = KU + 2;            // transposed half tiles: padded row (complex)
 constexpr int SLOT = TILE * TPITCH * 8;   // 4608 bytes
 constexpr int DX = 4;                     // vector slices in the ring
@@ -348,7 +333,7 @@ k_subst_stream(const STask* __restrict__ tasks, const int* __restrict__ off, int
             else if (tk.mode == BB) ok = run_task<RC, BB>(tk, jb, ts, xs, u, l, abort, polls, first);
             else {
                 ok = first();
-                float2* z = (tk.mode == ZERO_X ? jb.x : jb.acc) + (long long)(tk.own0 + tk.row0) * RC;
+                float2* z = (tk.mode == ST_ZERO_X ? jb.x : jb.acc) + (long long)(tk.own0 + tk.row0) * RC;
                 for (int e = l; ok && e < tk.nrows * RC / 2; e += 32) ((float4*)z)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
         }
@@ -407,12 +392,10 @@ void launch_stream(const StreamPlan& p, const void* jobs, int ldc, unsigned* syn
     }
 }
 
-// Phases, tasks and their blocks for the active products `prods` (mode, level, node of a job).
-void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vector<StreamProduct>& prods, int H,
-                  StreamPlan& plan) {
-    int sms = 0;
-    HZ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx.device));
-    const int G = sms, V = G * SW;
+// Phases, tasks and their warps for the active products `prods` (mode, level, node of a job).
+StreamLists stream_lists(const Ctx& ctx, const std::vector<int>& layers, const std::vector<StreamProduct>& prods, int H,
+                         int warps) {
+    const int V = warps;
     // phase of a product: FB by level, FA, (clearing acc), BB, BA by level downwards
     const int PFA = std::max(1, H), PZ = PFA + 1, PBB = PFA + 2;
     std::vector<std::vector<const StreamProduct*>> phases(PBB + 1 + H);
@@ -456,7 +439,7 @@ void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vec
                 s.store = whole;
                 if ((mode == FA || mode == BB) && !whole) {
                     STask z = s;
-                    z.mode = mode == FA ? ZERO_X : ZERO_ACC;
+                    z.mode = mode == FA ? ST_ZERO_X : ST_ZERO_ACC;
                     ts[mode == FA ? 0 : PZ].push_back(z);
                 }
                 for (int k = ub; k < ue; k += len) {
@@ -478,8 +461,8 @@ void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vec
     for (auto& ph : ts) {
         if (ph.empty()) continue;
         std::stable_sort(ph.begin(), ph.end(), [](const STask& a, const STask& c) { return a.nunits > c.nunits; });
-        // longest first to the least loaded warp (warp v in block v % G, so the first G tasks go to
-        // different SMs); a task's fixed cost counts as two half tiles
+        // longest first to the least loaded warp (warp v in block v % grid, so the first `grid` tasks go
+        // to different SMs); a task's fixed cost counts as two half tiles
         dealt.emplace_back(V);
         std::priority_queue<std::pair<long long, int>, std::vector<std::pair<long long, int>>, std::greater<>> load;
         for (int g = 0; g < V; ++g) load.push({0, g});
@@ -490,17 +473,25 @@ void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vec
             load.push({ld + s.nunits + 2, g});
         }
     }
-    std::vector<STask> all;   // by warp, then phase: a warp walks one contiguous list
-    std::vector<int> off;
+    StreamLists out;   // by warp, then phase: a warp walks one contiguous list
     for (int g = 0; g < V; ++g)
         for (const auto& ph : dealt) {
-            off.push_back((int)all.size());
-            all.insert(all.end(), ph[g].begin(), ph[g].end());
+            out.off.push_back((int)out.tasks.size());
+            out.tasks.insert(out.tasks.end(), ph[g].begin(), ph[g].end());
         }
-    off.push_back((int)all.size());
-    all.push_back(STask{});   // read ahead, never run
-    plan.nph = (int)dealt.size();
-    plan.grid = G;
+    out.off.push_back((int)out.tasks.size());
+    out.tasks.push_back(STask{});   // read ahead, never run
+    out.nph = (int)dealt.size();
+    return out;
+}
+
+void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vector<StreamProduct>& prods, int H,
+                  StreamPlan& plan) {
+    int sms = 0;
+    HZ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx.device));
+    const StreamLists ls = stream_lists(ctx, layers, prods, H, sms * SW);
+    plan.nph = ls.nph;
+    plan.grid = sms;
     auto up = [&](const void* src, size_t bytes) -> void* {
         void* d = nullptr;
         if (cudaMalloc(&d, std::max<size_t>(16, bytes)) != cudaSuccess) {
@@ -511,8 +502,8 @@ void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vec
         HZ_CUDA(cudaStreamSynchronize(ctx.stream));
         return d;
     };
-    plan.d_tasks = up(all.data(), all.size() * sizeof(STask));
-    plan.d_off = (int*)up(off.data(), off.size() * sizeof(int));
+    plan.d_tasks = up(ls.tasks.data(), ls.tasks.size() * sizeof(STask));
+    plan.d_off = (int*)up(ls.off.data(), ls.off.size() * sizeof(int));
 }
 
 }  // namespace hz

@@ -43,14 +43,13 @@
 #include "hz_ctx.cuh"
 #include "hz_solve.cuh"
 #include "tc_common.cuh"
+#include "subst_items.cuh"
 
 namespace hz {
 
 namespace {
 
 using namespace tcc;
-
-enum { FA = 0, FB = 1, BA = 2, BB = 3 };
 
 // Sizes of one ring stage for NT columns.  NT <= 64 runs the wide form of the MMAs (the output's
 // two halves side by side, three vector blocks per term); NT = 128 would need 6 x 8 KB of vector
@@ -96,96 +95,6 @@ __device__ __forceinline__ void read_acc(uint32_t tm, int c0, uint32_t (&vr)[16]
         }
     }
 }
-
-// One work item: 128 output rows (tiles o0 .. o0+3) x NT columns of one node product, reduction
-// tiles [kbeg, kend).
-struct Item {
-    JobDev<float2> jb;
-    NodeDev nd;
-    int col0, o0, nout_t, nrows_out, nrows_k, kbeg, kend, nst;
-    bool unique;
-};
-
-template <int NT, int MODE>
-__device__ inline Item decode(const Task* tasks, const JobDev<float2>* jobs, long long item, int nchunks) {
-    Item it;
-    const Task tk = tasks[item / nchunks];
-    it.jb = jobs[tk.job];
-    it.nd = it.jb.nodes[tk.node];
-    const NodeDev& nd = it.nd;
-    it.col0 = (int)(item % nchunks) * NT;
-    it.o0 = tk.tile;
-    it.nout_t = (MODE == FB) ? nd.upd_t : nd.own_t;
-    it.nrows_out = (MODE == FB) ? nd.nupd : nd.nown;
-    it.nrows_k = (MODE == BA) ? nd.nupd : nd.nown;
-    it.kbeg = tk.k0;
-    const int kfull0 = (MODE == BB) ? it.o0 : 0;
-    const int kfull1 = (MODE == FA) ? min(it.o0 + 4, nd.own_t) : ((MODE == BA) ? nd.upd_t : nd.own_t);
-    it.kend = it.kbeg + tk.klen;
-    it.nst = tk.klen * 2;
-    it.unique = it.kbeg == kfull0 && it.kend == kfull1 && MODE != FB && MODE != BA;
-    return it;
-}
-
-// Vector rows a loader thread copies in stage s of an item (-1: beyond the node, zero-filled).
-// They are looked up one stage ahead, so that BA's gather through the update index list is not
-// on the copy's critical path.
-template <int NT> struct Vrows { int r[KC * NT / 2 / NLOAD]; };
-
-template <int NT, int MODE>
-__device__ inline Vrows<NT> stage_rows(const Item& it, int s, int t) {
-    Vrows<NT> v;
-    const int kt = it.kbeg + (s >> 1), hk = s & 1;
-    const int* upd = it.jb.upd_idx + it.nd.upd_off;
-#pragma unroll
-    for (int i = 0; i < KC * NT / 2 / NLOAD; ++i) {
-        const int k = (t + NLOAD * i) / (NT / 2);
-        const int rr = kt * TILE + hk * KC + k;
-        v.r[i] = -1;
-        if (rr < it.nrows_k) v.r[i] = (MODE == BA) ? upd[rr] : it.nd.own0 + rr;
-    }
-    return v;
-}
-
-// The four factor tiles of an item's current reduction tile, as one loader thread copies them: its
-// first 16 bytes of each (8 per stage: 4 tiles x 2, 2 KB apart as stored, 16 columns apart where used
-// transposed).  Pointers advance from tile to tile; forming every copy's address anew (triangular
-// index, 64-bit products) kept a loader warp at some 230 instructions a stage, which bound narrow tiles.
-template <int MODE> struct TilePtrs {
-    static constexpr bool TR = (MODE == BA || MODE == BB);
-    const char* p[4];
-    int kt, o0, nout_t;
-    long long step;   // bytes to the next reduction tile (BB: of the first one on)
-
-    __device__ __forceinline__ void init(const Item& it, int t) {
-        const NodeDev& nd = it.nd;
-        kt = it.kbeg;
-        o0 = it.o0;
-        nout_t = it.nout_t;
-        const int thr = TR ? (t >> 3) * 256 + (t & 7) * 16 : t * 16;
-#pragma unroll
-        for (int oi = 0; oi < 4; ++oi) {
-            const int o = o0 + oi;
-            long long toff;
-            if (MODE == FA) toff = nd.linv_off + tri_idx(o, kt);
-            else if (MODE == FB) toff = nd.l21_off + (long long)o * nd.own_t + kt;
-            else if (MODE == BA) toff = nd.l21_off + (long long)kt * nd.own_t + o;
-            else toff = nd.linv_off + tri_idx(kt, o);
-            p[oi] = (const char*)(it.jb.fac + toff * TILE2) + thr;
-        }
-        step = (MODE == BA ? (long long)nd.own_t : MODE == BB ? (long long)kt + 1 : 1LL) * (TILE2 * 8);
-    }
-    __device__ __forceinline__ void next() {
-#pragma unroll
-        for (int oi = 0; oi < 4; ++oi) p[oi] += step;
-        ++kt;
-        if (MODE == BB) step += TILE2 * 8;
-    }
-    __device__ __forceinline__ bool exists(int oi) const {
-        const int o = o0 + oi;
-        return o < nout_t && (MODE != FA || kt <= o) && (MODE != BB || kt >= o);
-    }
-};
 
 // Loader part of stage s of an item: the four factor tiles' 16-column halves and 16 vector rows.
 template <int NT, int MODE>
@@ -328,15 +237,6 @@ __device__ inline void write_pair(const Item& it, long long base, int c, float4 
         if (it.unique) *dst = y;
         else atomicAdd(dst, y);
     }
-}
-
-// global offset (row x ldc + chunk column) of local output row r of an item, -1 if absent
-template <int MODE>
-__device__ inline long long row_base(const Item& it, int r, int ldc) {
-    const int row = it.o0 * TILE + r;
-    if ((it.o0 + (r >> 5)) >= it.nout_t || row >= it.nrows_out) return -1;
-    const int* upd = it.jb.upd_idx + it.nd.upd_off;
-    return ((MODE == FB) ? (long long)upd[row] : (long long)(it.nd.own0 + row)) * ldc + it.col0;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -530,9 +430,10 @@ template <int NT> struct PLayout {
     static constexpr bool SEP = NT == 32;
     static constexpr int CD = NT <= 64 ? 4 : 2;                    // converted operands' ring depth
     static constexpr int RD = NT == 32 ? 6 : NT == 64 ? 4 : 2;     // raw ring depth
-    // A converter group must have filled a ring slot's previous stage itself: a parity wait tells only
-    // the last phase from the one before, so it may not be reached while an older use is still open.
-    // Two groups take alternate stages, so both depths are even.
+    // Two converter groups take alternate stages.  A parity wait tells only the last phase from the one
+    // before, so nobody may reach it while an older use of the slot is still open.  With even depths a slot
+    // is one group's alone and the group's own previous wait on it has closed that use; with an odd
+    // depth it would follow only from the MMAs' commits arriving in the order of the stages.
     static_assert(CD % 2 == 0 && RD % 2 == 0, "a ring slot belongs to one converter group");
     static constexpr int CONV = TA ? 6 * RG::X_MAT : RG::CONV;
     static constexpr int NEPI = 128;                       // epilogue threads (4 warps)

@@ -23,7 +23,7 @@ constexpr long long WAIT_LIMIT = 1LL << 26;            // polls of one mbarrier 
 constexpr unsigned long long WAIT_NS = 2000000000ull;  // ... and at most 2 s of wall time
 constexpr int NLOAD = 128, NCONV = 256;                // loader and converter threads
 
-__device__ __forceinline__ long long tri_idx(int rt, int ct) { return (long long)rt * (rt + 1) / 2 + ct; }
+__host__ __device__ __forceinline__ long long tri_idx(int rt, int ct) { return (long long)rt * (rt + 1) / 2 + ct; }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
