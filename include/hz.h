@@ -74,9 +74,10 @@ typedef struct {
                             pass solves to 0.1 refine_tol / (its starting volume residual), capped at 0.1 */
     int32_t restart;     /* Krylov dimension before restart (default 12) */
     int32_t max_iter;    /* total GMRES iterations cap (default 100) */
-    double refine_tol;   /* mixed mode: refine until ||S f - A u|| <= refine_tol ||S f|| (default 1e-9).  A pass
-                            is added while the residual is above half of it, above a tenth of it where no
-                            correction has been made yet, so that a borderline pass is not the last one */
+    double refine_tol;   /* mixed mode: refine until ||S f - A u|| <= refine_tol ||S f|| (default 1e-9).  With
+                            the residual below it but above half of it (a tenth where no correction has
+                            been made yet) one pass more is tried, so that a borderline pass is not the
+                            last one, and kept only if it lowers the residual */
     int32_t max_refine;  /* mixed mode: maximum defect-correction passes (default 3) */
     int32_t krylov;      /* Krylov solver on the trace system: 0 GMRES(restart) (default), 1 Bi-CGSTAB
                             (two products P M_pol per iteration, six trace vectors per column instead
@@ -85,7 +86,7 @@ typedef struct {
 
 typedef struct {
     int32_t iters;         /* GMRES iterations of the last pass */
-    int32_t refinements;   /* defect-correction passes done (mixed mode) */
+    int32_t refinements;   /* defect-correction passes done (mixed mode), a dropped one included */
     double trace_relres;   /* final preconditioned relative residual estimate of GMRES */
     double volume_relres;  /* ||S f - A u|| / ||S f|| in FP64 (computed when refining or requested) */
     float ms_total;        /* device time of the whole call for this batch, milliseconds */

@@ -245,17 +245,25 @@ void do_solve(Ctx& c, const double2* rhs, int R, double2* u, const hz_solve_opts
                 d2h(c, hn.data(), norms, 2 * R * sizeof(double));
                 for (int r = 0; r < R; ++r) g2[r] = hn[2 * r + 1];
                 auto relres = [&](int r) { return g2[r] > 0 ? std::sqrt(hn[2 * r] / g2[r]) : 0.0; };
+                auto worst_relres = [&]() {
+                    double w = 0.0;
+                    for (int r = 0; r < R; ++r) w = std::max(w, std::isfinite(relres(r)) ? relres(r) : INFINITY);
+                    return w;
+                };
                 int passes = 0;
+                bool tried = false;   // the pass that was not needed for refine_tol has been made
                 for (;;) {
-                    double worst = 0.0;
-                    for (int r = 0; r < R; ++r) worst = std::max(worst, relres(r));
+                    const double worst = worst_relres();
                     if (!std::isfinite(worst)) { st_out = HZ_ERR_NONFINITE; break; }
                     // stop with some room below refine_tol.  The solution is some 10 times further off than
                     // its residual, and whether a first pass lands just below or just above the
                     // tolerance is up to the rounding of its local solves: a solution that was not
                     // corrected then has an error 100 times that of one that was.  So an uncorrected one
-                    // is accepted at a tenth of the tolerance, a corrected one at half of it.
-                    if (worst <= (passes == 0 ? 0.1 : 0.5) * o.refine_tol || passes >= o.max_refine) break;
+                    // is accepted at a tenth of the tolerance, a corrected one at half of it.  Between
+                    // there and refine_tol one pass more is tried, and kept only if it lowers the residual:
+                    // where FP64 goes no further, the solution at hand stands.
+                    if (worst <= (passes == 0 ? 0.1 : 0.5) * o.refine_tol || tried || passes >= o.max_refine) break;
+                    tried = worst <= o.refine_tol;
                     // defect correction: A du = r with the mixed path, u += du.  The correction
                     // needs the digits that bring the residual below refine_tol, with a factor 10
                     // to spare: its Krylov tolerance is 0.1 refine_tol / (current residual), never
@@ -264,15 +272,24 @@ void do_solve(Ctx& c, const double2* rhs, int R, double2* u, const hz_solve_opts
                     hz_solve_opts o2 = o;
                     o2.gmres_tol = std::min(1e-1, 0.1 * o.refine_tol / std::max(worst, 1e-300));
                     krylov_solve<float2>(c, res, false, R, du, o2, inf2.data());
-                    k_axpy_vol<<<cdiv((long long)R * N3, 256), 256, 0, c.stream>>>(u, du, (long long)R * N3);
+                    // a pass that may be dropped again leaves u as it is and puts u + du into du
+                    double2* next = tried ? du : u;
+                    k_axpy_vol<<<cdiv((long long)R * N3, 256), 256, 0, c.stream>>>(next, tried ? u : du, (long long)R * N3);
                     HZ_CHECK_LAUNCH();
                     ++passes;
                     for (int r = 0; r < R; ++r) {
                         inf[r].iters = inf2[r].iters;
                         inf[r].iters_total += inf2[r].iters;
                     }
-                    op_volume_residual(c, rhs, true, u, R, res, norms);
+                    const std::vector<double> hn_before = hn;
+                    op_volume_residual(c, rhs, true, next, R, res, norms);
                     d2h(c, hn.data(), norms, 2 * R * sizeof(double));
+                    if (tried) {
+                        if (worst_relres() < worst)
+                            HZ_CUDA(cudaMemcpyAsync(u, du, (size_t)R * N3 * sizeof(double2), cudaMemcpyDeviceToDevice, c.stream));
+                        else
+                            hn = hn_before;
+                    }
                 }
                 for (int r = 0; r < R; ++r) {
                     inf[r].refinements = passes;
