@@ -88,8 +88,8 @@ __device__ __forceinline__ void convert_operand(const unsigned char* rb, const f
             im[j] = a.y;
         }
         float4 rh, ih;
-        rh.x = tf32_hi(re[0]); rh.y = tf32_hi(re[1]); rh.z = tf32_hi(re[2]); rh.w = tf32_hi(re[3]);
-        ih.x = tf32_hi(im[0]); ih.y = tf32_hi(im[1]); ih.z = tf32_hi(im[2]); ih.w = tf32_hi(im[3]);
+        rh.x = tf32_hi<3>(re[0]); rh.y = tf32_hi<3>(re[1]); rh.z = tf32_hi<3>(re[2]); rh.w = tf32_hi<3>(re[3]);
+        ih.x = tf32_hi<3>(im[0]); ih.y = tf32_hi<3>(im[1]); ih.z = tf32_hi<3>(im[2]); ih.w = tf32_hi<3>(im[3]);
         const int off = coff(row, 4 * kq);
         *(float4*)(cv + 0 * G_AMAT + off) = rh;
         *(float4*)(cv + 1 * G_AMAT + off) = make_float4(re[0] - rh.x, re[1] - rh.y, re[2] - rh.z, re[3] - rh.w);

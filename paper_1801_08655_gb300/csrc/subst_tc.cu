@@ -154,11 +154,11 @@ __device__ inline void convert_stage(const unsigned char* rb, unsigned char* cv,
             float hi[8];
             const uint32_t col = ta + ((uint32_t)(32 * oi) << 16) + 8 * kh;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) { hi[j] = tf32_hi(re[j]); re[j] -= hi[j]; }
+            for (int j = 0; j < 8; ++j) { hi[j] = tf32_hi<SPLIT>(re[j]); re[j] -= hi[j]; }
             tmem_st8(col, hi);
             if (SPLIT == 3) tmem_st8(col + KC, re);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) { hi[j] = tf32_hi(im[j]); im[j] -= hi[j]; }
+            for (int j = 0; j < 8; ++j) { hi[j] = tf32_hi<SPLIT>(im[j]); im[j] -= hi[j]; }
             tmem_st8(col + 2 * KC, hi);
             if (SPLIT == 3) tmem_st8(col + 3 * KC, im);
         }
@@ -178,8 +178,8 @@ __device__ inline void convert_stage(const unsigned char* rb, unsigned char* cv,
             re[2] = a1.x; im[2] = a1.y; re[3] = a1.z; im[3] = a1.w;
         }
         float4 rh, ih;
-        rh.x = tf32_hi(re[0]); rh.y = tf32_hi(re[1]); rh.z = tf32_hi(re[2]); rh.w = tf32_hi(re[3]);
-        ih.x = tf32_hi(im[0]); ih.y = tf32_hi(im[1]); ih.z = tf32_hi(im[2]); ih.w = tf32_hi(im[3]);
+        rh.x = tf32_hi<SPLIT>(re[0]); rh.y = tf32_hi<SPLIT>(re[1]); rh.z = tf32_hi<SPLIT>(re[2]); rh.w = tf32_hi<SPLIT>(re[3]);
+        ih.x = tf32_hi<SPLIT>(im[0]); ih.y = tf32_hi<SPLIT>(im[1]); ih.z = tf32_hi<SPLIT>(im[2]); ih.w = tf32_hi<SPLIT>(im[3]);
         const int off = coff(row, 4 * kq);
         *(float4*)(cv + 0 * RG::A_MAT + off) = rh;
         *(float4*)(cv + 2 * RG::A_MAT + off) = ih;
@@ -195,8 +195,8 @@ __device__ inline void convert_stage(const unsigned char* rb, unsigned char* cv,
 #pragma unroll
         for (int j = 0; j < 4; ++j) { float2 a = src[(4 * kq + j) * NT + n]; re[j] = a.x; im[j] = a.y; }
         float4 rh, ih;
-        rh.x = tf32_hi(re[0]); rh.y = tf32_hi(re[1]); rh.z = tf32_hi(re[2]); rh.w = tf32_hi(re[3]);
-        ih.x = tf32_hi(im[0]); ih.y = tf32_hi(im[1]); ih.z = tf32_hi(im[2]); ih.w = tf32_hi(im[3]);
+        rh.x = tf32_hi<SPLIT>(re[0]); rh.y = tf32_hi<SPLIT>(re[1]); rh.z = tf32_hi<SPLIT>(re[2]); rh.w = tf32_hi<SPLIT>(re[3]);
+        ih.x = tf32_hi<SPLIT>(im[0]); ih.y = tf32_hi<SPLIT>(im[1]); ih.z = tf32_hi<SPLIT>(im[2]); ih.w = tf32_hi<SPLIT>(im[3]);
         const int off = (TA ? 0 : 4 * RG::A_MAT) + coff(n, 4 * kq);
         const float4 rl = make_float4(re[0] - rh.x, re[1] - rh.y, re[2] - rh.z, re[3] - rh.w);
         const float4 il = make_float4(im[0] - ih.x, im[1] - ih.y, im[2] - ih.z, im[3] - ih.w);

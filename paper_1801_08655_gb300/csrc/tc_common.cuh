@@ -38,9 +38,17 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
 // byte offset of (row, k) in a [rows x KC] K-major core-matrix operand (4-byte elements)
 __device__ __forceinline__ int coff(int row, int k) { return (row >> 3) * SBO + (k >> 2) * LBO + (row & 7) * 16 + (k & 3) * 4; }
 
-// v rounded to TF32 (10 mantissa bits), to nearest with ties away from zero, in two integer operations
-__device__ __forceinline__ float tf32_hi(float v) {
-    return __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xffffe000u);
+// v rounded to TF32 (10 mantissa bits), to nearest with ties away from zero.  With three terms (SPLIT = 3)
+// in two integer operations, which carry a NaN into the sign bit or to infinity; the low term v - hi is
+// then the NaN, and the product gets it from there.  The single term stands alone and keeps its NaN.
+template <int SPLIT> __device__ __forceinline__ float tf32_hi(float v) {
+    if constexpr (SPLIT == 3) {
+        return __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xffffe000u);
+    } else {
+        uint32_t r;
+        asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(v));
+        return __uint_as_float(r);
+    }
 }
 
 // 16-byte asynchronous global->shared copy; src_bytes = 0 zero-fills without reading
