@@ -488,6 +488,7 @@ void factor_layers(Ctx& ctx) {
     // the L21 and Schur products of large complex64 fronts run on the tensor cores
     const bool use_tc = sizeof(C) == 8 && ctx.factor_tc_min_upd > 0;
     try {
+        if (use_tc) front_gemm_allow_smem();
         for (int g0 = 0; g0 < L; g0 += G) {
             const int g1 = std::min(L, g0 + G);
             HZ_CUDA(cudaMemsetAsync(arena, 0, (size_t)per_layer * (g1 - g0), st));

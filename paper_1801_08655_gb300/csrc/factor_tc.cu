@@ -305,6 +305,11 @@ k_front_gemm(const GemmItem* __restrict__ items, const FrontGemmDesc* __restrict
 
 bool front_gemm_eligible(int nown, int nupd, int min_upd) { return nupd >= min_upd && nown >= TILE; }
 
+void front_gemm_allow_smem() {
+    for (auto* kern : {k_front_gemm<GEMM_L21>, k_front_gemm<GEMM_SCHUR>, k_front_gemm<GEMM_M21>})
+        HZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM));
+}
+
 // Work items of the three products for the given fronts (longest reductions first).
 void front_gemm_items(const std::vector<FrontGemmDesc>& fr, std::vector<GemmItem>& l21, std::vector<GemmItem>& schur,
                       std::vector<GemmItem>& m21) {
@@ -332,12 +337,7 @@ void front_gemm_items(const std::vector<FrontGemmDesc>& fr, std::vector<GemmItem
 void launch_front_gemm(int mode, const GemmItem* d_items, long long n, const FrontGemmDesc* d_fronts, int* flag,
                        long long polls, cudaStream_t st) {
     if (n <= 0) return;
-    static bool attr[3] = {false, false, false};
     auto* kern = mode == GEMM_L21 ? k_front_gemm<GEMM_L21> : mode == GEMM_SCHUR ? k_front_gemm<GEMM_SCHUR> : k_front_gemm<GEMM_M21>;
-    if (!attr[mode]) {
-        HZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM));
-        attr[mode] = true;
-    }
     for (long long b0 = 0; b0 < n; b0 += 65535LL * 16) {
         const unsigned grid = (unsigned)std::min<long long>(n - b0, 65535LL * 16);
         kern<<<grid, G_THREADS, G_SMEM, st>>>(d_items + b0, d_fronts, flag, polls);

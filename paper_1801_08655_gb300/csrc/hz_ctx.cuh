@@ -58,6 +58,7 @@ struct Batch {
     int sparse = 0;                             // products skipped away from the interface planes (get_batch)
     int job_cols = 0;                           // columns per job when per-block sparsity splits each
                                                 // layer's columns into jobs (0: one job per layer, ldc wide)
+    int sms = 1;                                // of the handle's device (blocks of a persistent launch)
     long long wait_polls = 1LL << 26;           // poll limit of the tensor-core kernels' pipeline waits
     std::vector<long long> pair_off[4], pair_cnt[4];  // tensor-core tasks: two output tiles each
     bool stream = false;                        // runs as one cooperative launch (plan below)
@@ -275,6 +276,7 @@ struct FrontGemmDesc {
 };
 struct GemmItem { int front, ti, tj, nst; };   // 128 x 128 output tile (ti, tj), pipeline stages
 bool front_gemm_eligible(int nown, int nupd, int min_upd);
+void front_gemm_allow_smem();   // their shared memory, on the current device
 void front_gemm_items(const std::vector<FrontGemmDesc>& fronts, std::vector<GemmItem>& l21,
                       std::vector<GemmItem>& schur, std::vector<GemmItem>& m21);
 void launch_front_gemm(int mode, const GemmItem* d_items, long long n, const FrontGemmDesc* d_fronts, int* flag,

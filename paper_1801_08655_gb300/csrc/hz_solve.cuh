@@ -9,6 +9,9 @@ namespace hz {
 int chunk_cols(bool is_double, int ncols);
 int tc_columns(int ldc);   // tensor-core column tile for this leading dimension (0: not usable)
 void launch_level_tc(const Batch& b, int h, int mode, int ldc, int* flag, cudaStream_t st);
+// More than the default 48 KiB of shared memory for a batch's tensor-core kernels, on the current device (a
+// kernel's attribute is the device's, so nothing remembers that it has been set); outside captures
+void prepare_tc(const Batch& b, int ldc);
 int padded_ldc(bool is_double, int ncols);
 // one-launch substitution of complex64 blocks (subst_stream.cu): usable for this leading dimension;
 // task lists of a batch's active products; the launch (sync: two counters, zero between launches)
@@ -37,7 +40,7 @@ struct StreamLists {
 };
 StreamLists stream_lists(const Ctx& ctx, const std::vector<int>& layers, const std::vector<StreamProduct>& prods, int H,
                          int warps);
-void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vector<StreamProduct>& prods, int H,
+void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vector<StreamProduct>& prods, int H, int ldc,
                   StreamPlan& plan);
 void launch_stream(const StreamPlan& p, const void* jobs, int ldc, unsigned* sync, int* flag, long long polls,
                    cudaStream_t st);

@@ -773,12 +773,14 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
     b.sparse = sparse;
     b.wait_polls = ctx.tc_wait_polls;
     b.stream = stream;
+    HZ_CUDA(cudaDeviceGetAttribute(&b.sms, cudaDevAttrMultiProcessorCount, ctx.device));
     // per-block sparsity: job j * nblk + q is block q (columns [q * job_cols, (q + 1) * job_cols))
     // of layer j; the caller has checked that the blocks tile the columns in whole chunks
     const int nblk = block_count(sparse);
     if (nblk > 1 && (ncols % nblk != 0 || (ncols / nblk) % 64 != 0 || ldc != ncols))
         throw Error{HZ_ERR_ARG, "per-block sparsity needs column blocks of a multiple of 64"};
     b.job_cols = nblk > 1 ? ncols / nblk : 0;
+    if (tc) prepare_tc(b, ldc);
     const bool m21 = has_m21<C>;
     BatchLists ls = batch_lists(ctx, layers, sizeof(C), KS, tc, KS_tc, min_t, sparse, stream);
     const int H = b.H = ls.H;
@@ -840,7 +842,7 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
                 b.alg_bytes += b.lvl_bytes[k][mode][h];
                 b.flops_per_col += b.lvl_flops[k][mode][h];
             }
-    if (stream) build_stream(ctx, layers, ls.prods, H, b.plan);
+    if (stream) build_stream(ctx, layers, ls.prods, H, ldc, b.plan);
     for (int w = 0; w < 2; ++w) {
         std::vector<ZeroDev>& zd = zero_rows[w];
         if (!m21)

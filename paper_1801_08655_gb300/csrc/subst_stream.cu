@@ -362,11 +362,6 @@ k_subst_stream(const STask* __restrict__ tasks, const int* __restrict__ off, int
 }
 
 template <int RC> void launch_rc(const StreamPlan& p, const void* jobs, unsigned* sync, int* flag, long long polls, cudaStream_t st) {
-    static bool attr = false;
-    if (!attr) {
-        HZ_CUDA(cudaFuncSetAttribute(k_subst_stream<RC>, cudaFuncAttributeMaxDynamicSharedMemorySize, SLayout<RC>::TOTAL));
-        attr = true;
-    }
     const STask* tasks = (const STask*)p.d_tasks;
     const int* off = p.d_off;
     int nph = p.nph;
@@ -375,6 +370,19 @@ template <int RC> void launch_rc(const StreamPlan& p, const void* jobs, unsigned
     HZ_CUDA(cudaLaunchCooperativeKernel((const void*)k_subst_stream<RC>, dim3(p.grid), dim3(32 * SW), args,
                                         (size_t)SLayout<RC>::TOTAL, st));
     HZ_CHECK_LAUNCH();
+}
+
+// the kernel's shared memory, on the current device; outside captures
+template <int RC> void allow_smem() {
+    HZ_CUDA(cudaFuncSetAttribute(k_subst_stream<RC>, cudaFuncAttributeMaxDynamicSharedMemorySize, SLayout<RC>::TOTAL));
+}
+void allow_smem(int ldc) {
+    switch (ldc) {
+        case 2: allow_smem<2>(); break;
+        case 4: allow_smem<4>(); break;
+        case 8: allow_smem<8>(); break;
+        default: allow_smem<16>(); break;
+    }
 }
 
 }  // namespace
@@ -485,10 +493,11 @@ StreamLists stream_lists(const Ctx& ctx, const std::vector<int>& layers, const s
     return out;
 }
 
-void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vector<StreamProduct>& prods, int H,
+void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vector<StreamProduct>& prods, int H, int ldc,
                   StreamPlan& plan) {
     int sms = 0;
     HZ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx.device));
+    allow_smem(ldc);
     const StreamLists ls = stream_lists(ctx, layers, prods, H, sms * SW);
     plan.nph = ls.nph;
     plan.grid = sms;

@@ -657,42 +657,33 @@ k_subst_tcp(const Task* __restrict__ tasks, const JobDev<float2>* __restrict__ j
     if (w == mma_warp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(TCOLS));
 }
 
-int sm_count() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        HZ_CUDA(cudaGetDevice(&dev));
-        HZ_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
-    }
-    return n;
-}
-
 template <int NT, int MODE, int SPLIT>
 void launch_one(const Batch& b, const Task* tasks, long long n, const JobDev<float2>* jobs, int ldc, int* flag,
                 cudaStream_t st) {
     const int nchunks = (b.job_cols > 0 ? b.job_cols : ldc) / NT;
     const long long nitems = n * nchunks;
     if (b.tc_cfg == 1) {
-        static bool attr = false;
-        if (!attr) {
-            HZ_CUDA(cudaFuncSetAttribute(k_subst_tcp<NT, MODE, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         PLayout<NT>::TOTAL));
-            attr = true;
-        }
-        const long long grid = std::min<long long>(nitems, sm_count());
+        const long long grid = std::min<long long>(nitems, b.sms);
         k_subst_tcp<NT, MODE, SPLIT><<<(unsigned)grid, PLayout<NT>::NTHREADS, PLayout<NT>::TOTAL, st>>>(
             tasks, jobs, ldc, nchunks, nitems, flag, b.wait_polls);
     } else {
-        static bool attr = false;
-        if (!attr) {
-            HZ_CUDA(cudaFuncSetAttribute(k_subst_tc<NT, MODE, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         OneLayout<NT>::TOTAL));
-            attr = true;
-        }
         k_subst_tc<NT, MODE, SPLIT><<<(unsigned)nitems, OneLayout<NT>::NTHREADS, OneLayout<NT>::TOTAL, st>>>(
             tasks, jobs, ldc, nchunks, flag, b.wait_polls);
     }
     HZ_CHECK_LAUNCH();
+}
+
+template <int NT, int MODE, int SPLIT> void allow_smem(int cfg) {
+    if (cfg == 1)
+        HZ_CUDA(cudaFuncSetAttribute(k_subst_tcp<NT, MODE, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, PLayout<NT>::TOTAL));
+    else
+        HZ_CUDA(cudaFuncSetAttribute(k_subst_tc<NT, MODE, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, OneLayout<NT>::TOTAL));
+}
+template <int NT, int SPLIT> void allow_smem_modes(int cfg) {
+    allow_smem<NT, FA, SPLIT>(cfg);
+    allow_smem<NT, FB, SPLIT>(cfg);
+    allow_smem<NT, BA, SPLIT>(cfg);
+    allow_smem<NT, BB, SPLIT>(cfg);
 }
 
 template <int NT, int SPLIT>
@@ -716,6 +707,19 @@ int tc_columns(int ldc) {
     if (ldc % 64 == 0) return 64;
     if (ldc % 32 == 0) return 32;
     return 0;
+}
+
+void prepare_tc(const Batch& b, int ldc) {
+    const int nt = tc_columns(b.job_cols > 0 ? b.job_cols : ldc);
+    if (b.split == 1) {
+        if (nt == 128) allow_smem_modes<128, 1>(b.tc_cfg);
+        else if (nt == 64) allow_smem_modes<64, 1>(b.tc_cfg);
+        else allow_smem_modes<32, 1>(b.tc_cfg);
+    } else {
+        if (nt == 128) allow_smem_modes<128, 3>(b.tc_cfg);
+        else if (nt == 64) allow_smem_modes<64, 3>(b.tc_cfg);
+        else allow_smem_modes<32, 3>(b.tc_cfg);
+    }
 }
 
 void launch_level_tc(const Batch& b, int h, int mode, int ldc, int* flag, cudaStream_t st) {
