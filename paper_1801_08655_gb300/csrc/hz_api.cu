@@ -418,8 +418,8 @@ hz_status hz_create_ex(const hz_grid* grid, const double* m, const double* b, do
         c.d_sz_n = dev_copy(szn); c.d_isz_h = dev_copy(iszh);
         c.d_m = dev_copy(std::vector<double>(m, m + N3));
         if (b) c.d_b = dev_copy(std::vector<double>(b, b + N3));
-        c.d_flag = (int*)dev_alloc(4 * sizeof(int));
-        HZ_CUDA(cudaMemset(c.d_flag, 0, 4 * sizeof(int)));
+        c.d_flag = (int*)dev_alloc(Ctx::FLAG_WORDS * sizeof(int));
+        HZ_CUDA(cudaMemset(c.d_flag, 0, Ctx::FLAG_WORDS * sizeof(int)));
         // layer partition: physical planes split evenly, earlier layers take the remainder;
         // layer 0 also owns the top PML planes, layer L-1 the bottom ones
         // nested-dissection leaf size (cells); HZ_LEAF overrides.  256-cell leaves give the
@@ -674,8 +674,8 @@ hz_status hz_create_shared(hz_handle* src, void* stream, hz_handle** out) {
         c.factored = true;
         c.owns_shared = false;
         c.stream = (cudaStream_t)stream;
-        c.d_flag = (int*)dev_alloc(4 * sizeof(int));
-        HZ_CUDA(cudaMemset(c.d_flag, 0, 4 * sizeof(int)));
+        c.d_flag = (int*)dev_alloc(Ctx::FLAG_WORDS * sizeof(int));
+        HZ_CUDA(cudaMemset(c.d_flag, 0, Ctx::FLAG_WORDS * sizeof(int)));
         HZ_CUDA(cudaDeviceSynchronize());
         *out = h;
         return HZ_OK;

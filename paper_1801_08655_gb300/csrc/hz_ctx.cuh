@@ -204,7 +204,10 @@ struct Ctx {
     double2 *d_sz_n = nullptr, *d_isz_h = nullptr;
     double* d_m = nullptr;
     double* d_b = nullptr;   // b = 1/rho on the global grid, nullptr for constant density
-    int* d_flag = nullptr;   // device error flags: [0] tiny pivot
+    // device words: [0] tiny pivot, [1] a wait gave up, [2], [3] barrier counters of the one-launch
+    // substitution, from FLAG_ZEROS on the cleared block of stream_fits
+    static constexpr int FLAG_ZEROS = 32, FLAG_WORDS = 64;
+    int* d_flag = nullptr;
     bool factored = false;
     bool owns_shared = true;  // false for handles that borrow another handle's factors (hz_create_shared)
     long long workspace_bytes = 0;
@@ -235,6 +238,7 @@ struct Ctx {
     int tc_mode = 2;        // tensor-core substitution (complex64, >= 64 columns): 0 never, 1 always,
                             // 2 when the autotuner measures it faster for the batch signature
     bool one_launch = true; // complex64 substitutions of at most 16 columns as one launch (HZ_ONE_LAUNCH)
+    std::map<int, bool> one_launch_fits;   // by leading dimension: the device holds that launch's grid
     int tc_ks = 4;          // split-K (factor tiles per block) of small tensor-core batches
     int tc_min_tiles = 8;   // output tiles a node product needs to run on the tensor cores
     int tc_cfg = 0;         // untuned tensor-core kernel: 0 one block per work item, 1 persistent (HZ_TC_CFG)

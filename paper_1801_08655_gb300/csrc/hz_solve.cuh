@@ -13,9 +13,12 @@ void launch_level_tc(const Batch& b, int h, int mode, int ldc, int* flag, cudaSt
 // kernel's attribute is the device's, so nothing remembers that it has been set); outside captures
 void prepare_tc(const Batch& b, int ldc);
 int padded_ldc(bool is_double, int ncols);
-// one-launch substitution of complex64 blocks (subst_stream.cu): usable for this leading dimension;
-// task lists of a batch's active products; the launch (sync: two counters, zero between launches)
+// one-launch substitution of complex64 blocks (subst_stream.cu): usable for this leading dimension; whether
+// the device holds its whole grid at once (asked before the first batch of a width; sets the kernel's
+// attributes); task lists of a batch's active products; the launch (sync: two counters, zero between
+// launches)
 bool stream_usable(int ldc);
+bool stream_fits(const Ctx& ctx, int ldc);
 // One task, as the host lays it out: the tile of step j sits at tile0 + j step + dstep j (j - 1) / 2.
 struct STask {
     long long tile0;
@@ -40,7 +43,7 @@ struct StreamLists {
 };
 StreamLists stream_lists(const Ctx& ctx, const std::vector<int>& layers, const std::vector<StreamProduct>& prods, int H,
                          int warps);
-void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vector<StreamProduct>& prods, int H, int ldc,
+void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vector<StreamProduct>& prods, int H,
                   StreamPlan& plan);
 void launch_stream(const StreamPlan& p, const void* jobs, int ldc, unsigned* sync, int* flag, long long polls,
                    cudaStream_t st);
@@ -81,6 +84,8 @@ struct BatchLists {
 };
 BatchLists batch_lists(const Ctx& ctx, const std::vector<int>& layers, size_t elem, int KS, bool tc, int KS_tc, int min_t,
                        int sparse, bool stream);
+// Whether a complex64 batch of this leading dimension and sparsity code runs as one launch.
+bool use_one_launch(Ctx& ctx, int ldc, int sparse);
 // Candidates that the tuner times for this leading dimension.  Host only.
 std::vector<Ctx::TuneChoice> tune_candidates(const Ctx& ctx, bool is_double, int ncols);
 

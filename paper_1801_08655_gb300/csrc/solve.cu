@@ -518,10 +518,15 @@ static bool tc_usable(const Ctx& ctx, int ldc) {
 }
 
 // Complex64 blocks of at most 16 columns run as one launch (subst_stream.cu): faster than the launches
-// per phase at every width, tree and layer set measured (24^3 to 64^3, one layer: 1.5-1.9x, all
-// layers: 1.3-1.7x), so nothing is timed for them.
-static bool use_one_launch(const Ctx& ctx, int ldc, int sparse) {
-    return ctx.one_launch && stream_usable(ldc) && block_count(sparse) == 1;
+// per phase at every width and size measured, so nothing is timed for them (substitution time, 2 / 4 / 8
+// / 16 columns, launches per phase over one launch; one layer: 64^3 1.6 1.8 1.9 1.6, 128^3 1.2 1.5 1.7 1.5,
+// 160^3 1.3 1.5 1.8 1.5; all layers: 64^3 1.3 1.5 1.8 1.5, 128^3 1.2 1.5 1.9 1.6, 160^3 1.2 1.5 1.9 1.6).  Where
+// the device does not hold the whole grid at once, the launches per phase are the way.
+bool use_one_launch(Ctx& ctx, int ldc, int sparse) {
+    if (!ctx.one_launch || !stream_usable(ldc) || block_count(sparse) != 1) return false;
+    auto it = ctx.one_launch_fits.find(ldc);
+    if (it == ctx.one_launch_fits.end()) it = ctx.one_launch_fits.emplace(ldc, stream_fits(ctx, ldc)).first;
+    return it->second;
 }
 
 static std::string tune_key(const Ctx& ctx, const std::vector<int>& layers, int ldc, int split, int sparse) {
@@ -842,7 +847,7 @@ Batch& get_batch_cfg(Ctx& ctx, const std::vector<int>& layers, int ncols, int KS
                 b.alg_bytes += b.lvl_bytes[k][mode][h];
                 b.flops_per_col += b.lvl_flops[k][mode][h];
             }
-    if (stream) build_stream(ctx, layers, ls.prods, H, ldc, b.plan);
+    if (stream) build_stream(ctx, layers, ls.prods, H, b.plan);
     for (int w = 0; w < 2; ++w) {
         std::vector<ZeroDev>& zd = zero_rows[w];
         if (!m21)

@@ -372,17 +372,32 @@ template <int RC> void launch_rc(const StreamPlan& p, const void* jobs, unsigned
     HZ_CHECK_LAUNCH();
 }
 
-// the kernel's shared memory, on the current device; outside captures
-template <int RC> void allow_smem() {
+// The kernel's shared memory on the current device, and whether a launch of `grid` blocks fits there at
+// once: by the occupancy, and by the launch itself (with no phases) where the context has fewer SMs than
+// the device.  `zeros`: 128 cleared bytes (they are zero again afterwards).  Outside captures.
+template <int RC> bool grid_fits(int grid, void* zeros, cudaStream_t st) {
     HZ_CUDA(cudaFuncSetAttribute(k_subst_stream<RC>, cudaFuncAttributeMaxDynamicSharedMemorySize, SLayout<RC>::TOTAL));
-}
-void allow_smem(int ldc) {
-    switch (ldc) {
-        case 2: allow_smem<2>(); break;
-        case 4: allow_smem<4>(); break;
-        case 8: allow_smem<8>(); break;
-        default: allow_smem<16>(); break;
+    int per_sm = 0;
+    HZ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_subst_stream<RC>, 32 * SW, SLayout<RC>::TOTAL));
+    if (per_sm < 1) return false;
+    const STask* tasks = (const STask*)zeros;
+    const int* off = (const int*)zeros;
+    int nph = 0;
+    const JobDev<float2>* jd = nullptr;
+    unsigned* sync = (unsigned*)zeros + 16;   // behind the one task that is read
+    int* flag = (int*)zeros + 18;
+    long long polls = 1;
+    void* args[] = {&tasks, &off, &nph, &jd, &sync, &flag, &polls};
+    const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_subst_stream<RC>, dim3(grid), dim3(32 * SW), args,
+                                                      (size_t)SLayout<RC>::TOTAL, st);
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported || e == cudaErrorNotPermitted) {
+        cudaGetLastError();
+        return false;
     }
+    HZ_CUDA(e);
+    HZ_CHECK_LAUNCH();
+    HZ_CUDA(cudaStreamSynchronize(st));
+    return true;
 }
 
 }  // namespace
@@ -493,11 +508,22 @@ StreamLists stream_lists(const Ctx& ctx, const std::vector<int>& layers, const s
     return out;
 }
 
-void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vector<StreamProduct>& prods, int H, int ldc,
+bool stream_fits(const Ctx& ctx, int ldc) {
+    int coop = 0, sms = 0;
+    HZ_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx.device));
+    HZ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx.device));
+    if (!coop) return false;
+    void* zeros = ctx.d_flag + Ctx::FLAG_ZEROS;
+    if (ldc == 2) return grid_fits<2>(sms, zeros, ctx.stream);
+    if (ldc == 4) return grid_fits<4>(sms, zeros, ctx.stream);
+    if (ldc == 8) return grid_fits<8>(sms, zeros, ctx.stream);
+    return grid_fits<16>(sms, zeros, ctx.stream);
+}
+
+void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vector<StreamProduct>& prods, int H,
                   StreamPlan& plan) {
     int sms = 0;
     HZ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx.device));
-    allow_smem(ldc);
     const StreamLists ls = stream_lists(ctx, layers, prods, H, sms * SW);
     plan.nph = ls.nph;
     plan.grid = sms;

@@ -436,6 +436,18 @@ int main(int argc, char** argv) {
             check_lists(c, sets[0], 8, ncols, 8, true, kst, 2, blocked_code(4, blocks));
             check_lists(c, sets[0], 8, ncols, 1 << 30, false, 1 << 30, 0, blocked_code(4, blocks));
         }
+    where = "route";   // a device that holds the grid at once takes the one launch, another the tuner's choice
+    for (int ldc : {2, 4, 8, 16}) {
+        c.one_launch_fits[ldc] = true;
+        CHECK(use_one_launch(c, ldc, 0) && use_one_launch(c, ldc, one_code[1]));
+        c.one_launch_fits[ldc] = false;
+        CHECK(!use_one_launch(c, ldc, 0) && !tune_candidates(c, false, ldc).empty());
+        c.one_launch_fits[ldc] = true;
+        c.one_launch = false;
+        CHECK(!use_one_launch(c, ldc, 0));
+        c.one_launch = true;
+    }
+    for (int ldc : {1, 32, 64, 128}) CHECK(!use_one_launch(c, ldc, 0));
     where = "fronts";
     for (int min_upd : {1, 128}) check_front_items(c, min_upd);
     std::printf("%lld tasks, %lld tensor-core stages, %lld half tiles\n", n_tasks, n_stages, n_units);

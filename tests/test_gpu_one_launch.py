@@ -51,3 +51,24 @@ def test_every_width_in_one_launch(shape, precision):
         assert rel(got, want) < TOL[precision], (R, rel(got, want))
     s.close()
     ref.close()
+
+
+def test_agrees_with_the_launches_per_phase(monkeypatch):
+    """Where the one launch is not taken (HZ_ONE_LAUNCH=0, or a device that cannot hold its whole grid), the
+    launches per phase give the same solves, with more launches."""
+    from paper_1801_08655_gb300 import build
+    build.build()
+    shape = (21, 24, 23)
+    one = one_layer(shape, "mixed")
+    monkeypatch.setenv("HZ_ONE_LAUNCH", "0")
+    per_phase = one_layer(shape, "mixed")
+    for R in (1, 4, 16):
+        g = sources(shape, R, R)
+        want = per_phase.layer_solve(0, g)
+        per_phase.profile_begin(detail=True)
+        per_phase.layer_solve(0, g)
+        per_phase.profile_end()
+        assert per_phase.profile_kernel(0)["launches"] > 4
+        assert rel(one.layer_solve(0, g), want) < 5e-6   # the same factors, other summation orders
+    one.close()
+    per_phase.close()
