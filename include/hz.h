@@ -113,10 +113,12 @@ void hz_default_opts(hz_precision prec, hz_solve_opts* opts);
  * Errors: HZ_ERR_ARG, HZ_ERR_NONFINITE (m), HZ_ERR_OOM, HZ_ERR_CUDA.
  * Environment variables read here (they change speed, never the solution beyond rounding):
  *   HZ_SUBST_TC       complex64 substitutions on the tcgen05 kernel: 0 never, 1 always (for
- *                     more than 16 columns), 2 (default) when the autotuner times it faster
+ *                     more than 16 columns; more than 32 on factors rounded from FP64), 2
+ *                     (default) when the autotuner times it faster
  *   HZ_ONE_LAUNCH=0   complex64 substitutions of at most 16 columns as one launch per phase and tree
  *                     level instead of one cooperative launch
- *   HZ_TC_MIN_TILES   default minimum output tiles of a tensor-core product (8)
+ *   HZ_TC_MIN_TILES   minimum output tiles of a tensor-core product: 8 where nothing is timed; the
+ *                     autotuner times 2, and the value set here beside it
  *   HZ_PRECOND_SPLIT  1: single-term TF32 tensor-core products inside the preconditioner
  *                     (default 3 terms, FP32-level)
  *   HZ_TC_CFG=1       with HZ_AUTOTUNE=0: the persistent tensor-core kernel (one block per SM

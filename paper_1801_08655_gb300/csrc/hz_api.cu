@@ -506,7 +506,10 @@ hz_status hz_create_ex(const hz_grid* grid, const double* m, const double* b, do
         if (const char* e = std::getenv("HZ_TC_KS")) c.tc_ks = std::max(1, std::atoi(e));
         if (const char* e = std::getenv("HZ_AUTOTUNE")) c.autotune = std::atoi(e) != 0;
         if (const char* e = std::getenv("HZ_GRAPHS")) c.use_graphs = std::atoi(e) != 0;
-        if (const char* e = std::getenv("HZ_TC_MIN_TILES")) c.tc_min_tiles = std::max(1, std::atoi(e));
+        if (const char* e = std::getenv("HZ_TC_MIN_TILES")) {
+            c.tc_min_tiles = std::max(1, std::atoi(e));
+            c.tc_min_set = true;
+        }
         // HZ_PRECOND_SPLIT=1: single-term TF32 tensor-core products inside the preconditioner
         if (const char* e = std::getenv("HZ_PRECOND_SPLIT")) c.precond_split = std::atoi(e) == 1 ? 1 : 3;
         if (const char* e = std::getenv("HZ_TC_CFG")) c.tc_cfg = std::atoi(e) == 0 ? 0 : 1;
@@ -666,7 +669,8 @@ hz_status hz_create_shared(hz_handle* src, void* stream, hz_handle** out) {
         c.d_sx_n = s.d_sx_n; c.d_isx_h = s.d_isx_h; c.d_sy_n = s.d_sy_n; c.d_isy_h = s.d_isy_h;
         c.d_sz_n = s.d_sz_n; c.d_isz_h = s.d_isz_h; c.d_m = s.d_m; c.d_b = s.d_b;
         c.one_launch = s.one_launch;
-        c.tc_mode = s.tc_mode; c.tc_ks = s.tc_ks; c.tc_min_tiles = s.tc_min_tiles; c.precond_split = s.precond_split; c.tc_cfg = s.tc_cfg;
+        c.tc_mode = s.tc_mode; c.tc_ks = s.tc_ks; c.tc_min_tiles = s.tc_min_tiles; c.tc_min_set = s.tc_min_set;
+        c.precond_split = s.precond_split; c.tc_cfg = s.tc_cfg;
         c.sparse_subst = s.sparse_subst;
         c.tc_wait_polls = s.tc_wait_polls;
         c.autotune = s.autotune; c.use_graphs = s.use_graphs;

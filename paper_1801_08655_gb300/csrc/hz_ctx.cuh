@@ -235,12 +235,13 @@ struct Ctx {
     struct TuneChoice { int KS, CC, tc, KS_tc, min_t, tc_cfg; };
     std::map<std::string, TuneChoice> tuned;
     std::vector<std::string> tune_log;
-    int tc_mode = 2;        // tensor-core substitution (complex64, >= 64 columns): 0 never, 1 always,
-                            // 2 when the autotuner measures it faster for the batch signature
+    int tc_mode = 2;        // tensor-core substitution (complex64, more than 16 columns; more than 32 on factors
+                            // rounded from FP64): 0 never, 1 always, 2 when the autotuner measures it faster
     bool one_launch = true; // complex64 substitutions of at most 16 columns as one launch (HZ_ONE_LAUNCH)
     std::map<int, bool> one_launch_fits;   // by leading dimension: the device holds that launch's grid
     int tc_ks = 4;          // split-K (factor tiles per block) of small tensor-core batches
-    int tc_min_tiles = 8;   // output tiles a node product needs to run on the tensor cores
+    int tc_min_tiles = 8;   // output tiles a node product needs to run on the tensor cores, untuned ...
+    bool tc_min_set = false;   // ... and, where the caller set it (HZ_TC_MIN_TILES), a candidate of the tuner
     int tc_cfg = 0;         // untuned tensor-core kernel: 0 one block per work item, 1 persistent (HZ_TC_CFG)
     int precond_split = 3;  // TF32 terms of the tensor-core products inside the preconditioner (3 or 1)
     long long tc_wait_polls = 1LL << 26;  // poll limit of the tensor-core pipeline waits (HZ_TC_WAIT_POLLS:

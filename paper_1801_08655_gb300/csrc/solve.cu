@@ -575,14 +575,16 @@ std::vector<Ctx::TuneChoice> tune_candidates(const Ctx& ctx, bool dbl, int ncols
                 if (!try_tc || ks == 8 || ks == (1 << 30)) cands.push_back({ks, cc, 0, 1 << 30, 0, 0});
     }
     if (try_tc) {
-        // every product of two output tiles or more (fewer never won); persistent kernel at all
+        // every product of two output tiles or more (4 and 8 never won), and what the caller set; persistent kernel at all
         // depths (a single layer's steps want 2-8 tiles a work item, 64^3 with 128 columns: 0.62 ms
         // at 4 against 0.88 at 16; all layers together 16 and more), one block per item at two
         std::vector<int> mts{2};
-        if (ctx.tc_min_tiles < 8 && ctx.tc_min_tiles != 2) mts.push_back(ctx.tc_min_tiles);
+        if (ctx.tc_min_set && ctx.tc_min_tiles != 2) mts.push_back(ctx.tc_min_tiles);
         for (int mt : mts) {
             // factors from FP64: the per-item kernel alone, whose hi x lo terms have accumulators of their
-            // own at every width (a 40^3 layer solve on 64 columns 2.5e-6 off, 1.0e-5 without)
+            // own at every width (a 40^3 layer solve on 64 columns 3.8e-6 off FP64, 1.0e-5 without).  The
+            // persistent kernel would take 0.7 to 1.0 of its time (64^3 layer, 64 columns 0.59 against 0.81 ms;
+            // 56^3, 128 columns 0.79 against 0.91); whoever keeps FP64-derived factors wants the digits.
             if (ctx.prec == HZ_PREC_MIXED)
                 for (int kstc : {2, 4, 8, 16, 1 << 30}) cands.push_back({8, cc0, 1, kstc, mt, 1});
             for (int kstc : {4, 1 << 30}) cands.push_back({8, cc0, 1, kstc, mt, 0});

@@ -448,6 +448,22 @@ int main(int argc, char** argv) {
         c.one_launch = true;
     }
     for (int ldc : {1, 32, 64, 128}) CHECK(!use_one_launch(c, ldc, 0));
+    where = "tuner";   // a minimum of output tiles that the caller set is timed, whatever its value
+    for (int ncols : {17, 64, 128})
+        for (int set : {1, 4, 8, 16}) {
+            auto has = [&](int t) {
+                for (auto& cd : tune_candidates(c, false, ncols))
+                    if (cd.tc && cd.min_t == t) return true;
+                return false;
+            };
+            c.prec = HZ_PREC_MIXED;
+            c.tc_min_tiles = set;
+            c.tc_min_set = true;
+            CHECK(has(set) && has(2));
+            c.tc_min_tiles = 8;
+            c.tc_min_set = false;
+            CHECK(!has(8) && has(2));
+        }
     where = "fronts";
     for (int min_upd : {1, 128}) check_front_items(c, min_upd);
     std::printf("%lld tasks, %lld tensor-core stages, %lld half tiles\n", n_tasks, n_stages, n_units);
