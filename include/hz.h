@@ -129,9 +129,10 @@ void hz_default_opts(hz_precision prec, hz_solve_opts* opts);
  *                     side skip the products of subtrees that hold none of a layer's interface
  *                     planes (3, default: forward and backward; 2: backward only; 0: never)
  *   HZ_FACTOR_PROFILE=1  time every factorization launch by kernel kind (hz_factor_report)
- *   HZ_TC_WAIT_POLLS  poll limit of the tensor-core kernels' pipeline waits (default 2^26, and
- *                     2 s of wall time); a tiny value makes them give up at once, which a solve
- *                     reports as HZ_ERR_TIMEOUT (the blocks still drain their own copies and MMAs)
+ *   HZ_TC_WAIT_POLLS  poll limit of the bounded waits in the tensor-core kernels and in the one-launch
+ *                     substitution (default 2^26, and 2 s of wall time); a tiny value makes them
+ *                     give up at once, which the call reports as HZ_ERR_TIMEOUT (the blocks still
+ *                     drain their own copies and MMAs)
  *   HZ_FACTOR_TC_MIN  complex64 fronts with at least this many update unknowns (default 128)
  *                     compute L21 and their Schur complement on the tensor cores; 0: never
  */
@@ -170,7 +171,7 @@ hz_status hz_factor(hz_handle* h);
  *   info  NULL or array of R entries, one per right-hand side (iters etc. of its column)
  * Errors: HZ_ERR_STATE (not factored), HZ_ERR_ARG, HZ_ERR_ADMISSION (workspace for R
  * does not fit), HZ_ERR_OOM, HZ_ERR_NONFINITE, HZ_ERR_NO_CONVERGENCE (u and info still written),
- * HZ_ERR_TIMEOUT (a tensor-core kernel's bounded wait gave up), HZ_ERR_CUDA.
+ * HZ_ERR_TIMEOUT (a bounded wait in a substitution gave up), HZ_ERR_CUDA.
  */
 hz_status hz_solve(hz_handle* h, const double* rhs, int32_t R, double* u,
                    const hz_solve_opts* opts, hz_solve_info* info);
@@ -226,7 +227,8 @@ const char* hz_last_error(const hz_handle* h);
 
 /* ------------------------------------------------------------------------------------
  * Introspection and stage-level entry points.  Each runs one step of the online path
- * on the device so that it can be checked on its own; none is needed for a solve.
+ * on the device so that it can be checked on its own; none is needed for a solve.  A bounded wait that
+ * gives up in one of their substitutions is HZ_ERR_TIMEOUT, as in hz_solve.
  * ------------------------------------------------------------------------------------ */
 
 /* Layer geometry of the layered decomposition (Formulation section, Fig. 1 and Eq. 6): owned

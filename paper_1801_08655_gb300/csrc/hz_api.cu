@@ -305,7 +305,7 @@ void do_solve(Ctx& c, const double2* rhs, int R, double2* u, const hz_solve_opts
     d2h(c, flags, c.d_flag, sizeof(flags));
     if (flags[1]) {
         HZ_CUDA(cudaMemset(c.d_flag + 1, 0, sizeof(int)));
-        throw Error{HZ_ERR_TIMEOUT, "a tensor-core substitution block gave up waiting on its MMAs"};
+        throw Error{HZ_ERR_TIMEOUT, WAIT_GAVE_UP};
     }
     HZ_CUDA(cudaEventRecord(e1, c.stream));
     HZ_CUDA(cudaEventSynchronize(e1));

@@ -48,6 +48,10 @@ void build_stream(const Ctx& ctx, const std::vector<int>& layers, const std::vec
 void launch_stream(const StreamPlan& p, const void* jobs, int ldc, unsigned* sync, int* flag, long long polls,
                    cudaStream_t st);
 
+// HZ_ERR_TIMEOUT of a substitution: a tensor-core block's pipeline wait, or a tile wait or phase barrier of
+// the one-launch kernel
+constexpr const char* WAIT_GAVE_UP = "a substitution block gave up on one of its bounded waits";
+
 // Sparsity of a batch: which planes of each layer carry the sources (forward code, bits 0-1) and
 // the read-outs (backward code, bits 2-3).  SP_ALL: anywhere (no product skipped); SP_BOTH: the
 // plane pairs next to both internal interfaces; SP_TOP / SP_BOT: the pair next to the top /

@@ -962,7 +962,7 @@ inline void check_waits(Ctx& ctx) {
     HZ_CUDA(cudaStreamSynchronize(ctx.stream));
     if (!flag) return;
     HZ_CUDA(cudaMemsetAsync(ctx.d_flag + 1, 0, sizeof(int), ctx.stream));
-    throw Error{HZ_ERR_TIMEOUT, "a substitution block gave up on one of its waits"};
+    throw Error{HZ_ERR_TIMEOUT, WAIT_GAVE_UP};
 }
 
 // run a freshly recorded operator once and release its descriptors

@@ -72,3 +72,22 @@ def test_agrees_with_the_launches_per_phase(monkeypatch):
         assert rel(one.layer_solve(0, g), want) < 5e-6   # the same factors, other summation orders
     one.close()
     per_phase.close()
+
+
+def test_give_up_leaves_the_counters_usable(tmp_path):
+    """On one handle: a wait that gives up is a status with a text that fits, the barrier counters are
+    zero afterwards, and the next application is right."""
+    import os
+    import shutil
+    import subprocess
+    from paper_1801_08655_gb300 import build
+    lib = build.build()
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    exe = str(tmp_path / "one_launch_give_up")
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "native", "one_launch_give_up.cu")
+    r = subprocess.run([nvcc, *build.ARCH, "-O2", "-std=c++17", "-I", build.INCLUDE, "-I", build.CSRC, src, "-o", exe,
+                        "-L", os.path.dirname(lib), "-lhz", "-Xlinker", "-rpath=" + os.path.dirname(lib)],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout + r.stderr
