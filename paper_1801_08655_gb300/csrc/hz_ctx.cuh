@@ -29,7 +29,7 @@ struct LayerCoef {
     double omega2, inv_h2;
 };
 
-// One vector to clear (launch_zero): 8-byte aligned pointer, a multiple of 8 bytes.
+// One vector to clear (launch_zero): 16-byte aligned, a multiple of 16 bytes (complex64 columns come in pairs).
 struct ZeroDev { void* p; long long bytes; };
 // Clears n vectors, the longest of max_bytes, in one launch.
 void launch_zero(const ZeroDev* d, int n, long long max_bytes, cudaStream_t st);
@@ -59,8 +59,8 @@ struct Batch {
     int job_cols = 0;                           // columns per job when per-block sparsity splits each
                                                 // layer's columns into jobs (0: one job per layer, ldc wide)
     int sms = 1;                                // of the handle's device (blocks of a persistent launch)
-    long long wait_polls = 1LL << 26;           // poll limit of the tensor-core kernels' pipeline waits
-    std::vector<long long> pair_off[4], pair_cnt[4];  // tensor-core tasks: two output tiles each
+    long long wait_polls = 1LL << 26;           // poll limit of the tensor-core and one-launch kernels' waits
+    std::vector<long long> pair_off[4], pair_cnt[4];  // tensor-core tasks: four output tiles each
     bool stream = false;                        // runs as one cooperative launch (plan below)
     StreamPlan plan;
     Task* d_tasks = nullptr;
@@ -244,8 +244,8 @@ struct Ctx {
     bool tc_min_set = false;   // ... and, where the caller set it (HZ_TC_MIN_TILES), a candidate of the tuner
     int tc_cfg = 0;         // untuned tensor-core kernel: 0 one block per work item, 1 persistent (HZ_TC_CFG)
     int precond_split = 3;  // TF32 terms of the tensor-core products inside the preconditioner (3 or 1)
-    long long tc_wait_polls = 1LL << 26;  // poll limit of the tensor-core pipeline waits (HZ_TC_WAIT_POLLS:
-                                          // a small value makes the waits give up, to test that path)
+    long long tc_wait_polls = 1LL << 26;  // poll limit of the tensor-core and one-launch kernels' waits
+                                          // (HZ_TC_WAIT_POLLS: a small value makes them give up, to test that)
     int sparse_subst = 3;   // skip substitution products away from the interface planes where the
                             // operator allows it (bit 0 forward, bit 1 backward; HZ_SPARSE)
     bool factor_prof = false;     // time every factorization launch by kernel kind (HZ_FACTOR_PROFILE=1)

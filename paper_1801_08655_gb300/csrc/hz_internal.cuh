@@ -74,7 +74,8 @@ struct NodeDev {            // device copy of what the solve kernels need per tr
     int pad_;
     long long upd_off;      // into the shape's upd_idx array
     long long linv_off;     // tile offset of packed lower-triangular L^{-1} (own_t*(own_t+1)/2 tiles)
-    long long l21_off;      // tile offset of L21 (upd_t x own_t tiles, row-tile major)
+    long long l21_off;      // tile offset of M21 = L21 L11^{-1} (complex64) or L21 (complex128): upd_t x
+                            // own_t tiles, row-tile major
 };
 
 struct Node {
@@ -151,8 +152,8 @@ template <class C> struct JobDev {
     const C* dinv;
     const NodeDev* nodes;
     const int* upd_idx;
-    C* acc;   // accumulator (forward) / scratch (backward)
-    C* x;     // solution
+    C* acc;   // right-hand side; complex64: the solution too, complex128: scratch of the backward pass
+    C* x;     // complex128: the solution; complex64: D^{-1} L^{-1} acc of every node
 };
 
 // One output tile (four on the tensor cores) of a node product over reduction tiles [k0, k0 + klen).

@@ -106,8 +106,8 @@ template <class C> void ensure_tuned(Ctx& ctx, const std::vector<int>& layers, i
 void free_batches(Ctx& ctx);
 
 // Forward/backward substitution for every job of the batch on ncols columns of the
-// layers' slot vectors (acc holds the right-hand side in elimination order on entry and
-// is clobbered; x receives the solution).
+// layers' slot vectors (acc holds the right-hand side in elimination order on entry; the solution is in
+// Ctx::result afterwards, the other vector is clobbered).
 template <class C> void substitute(Ctx& ctx, const Batch& b, int ncols, cudaStream_t st);
 
 // Online operators on polarized trace vectors [R][2][K][2][P] (complex128, device).

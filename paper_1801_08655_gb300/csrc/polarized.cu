@@ -52,9 +52,8 @@ template <class C> struct Inject {
 // through shared memory so that both sides are read and written along their contiguous index
 // (tile[a][b] with a pitch of 33 16-byte elements: conflict-free along either index).  What depends on the
 // cell alone (row, FP64 weight) is formed once per cell, by one warp beside the loads: formed per
-// element it was most of the FP64 work that bound them (64^3, 16 columns: volume source 172 us,
-// injection 28 us; a 64^3 solve with 16 columns 43.5 -> 40.9 ms with this and the sweeps' batched
-// clearing, 128^3 with 32 columns 932 -> 894 ms).  With fewer right-hand sides than lanes, a warp takes several cells at once.
+// element it was most of the FP64 work that bound them (64^3, 16 columns: volume source 172 -> 84 us,
+// injection 28 -> 13 us).  With fewer right-hand sides than lanes, a warp takes several cells at once.
 constexpr int IO_T = 32;
 
 // lanes along the right-hand sides of a tile: the smallest power of two that holds them

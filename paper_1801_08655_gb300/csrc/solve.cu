@@ -13,8 +13,9 @@
 // and the solution is left in acc.  That is 2 (H - 1) + 2 dependent phases for a tree of H levels
 // where L21 needs 4 H, with the same flops and factor bytes; the phases that leave the recursion
 // (half of them, and the ones with the shortest reductions) fill the GPU however few nodes a
-// level has.  Whole solves, L21 against M21: 24^3 with 1 column 2.60 -> 1.95 ms, 64^3 with 16
-// columns 99.3 -> 80.3 ms, with 128 columns 283 -> 204 ms.  Complex128 factors, whose products are bound by the FP64 pipe at any size, keep L21:
+// level has.  One layer as launches per phase, L21 against M21 (and clearing split rows alone): 24^3, 1
+// column 0.156 -> 0.093 ms; 64^3, 1 / 4 / 16 columns 0.432 -> 0.294, 0.498 -> 0.349, 0.776 -> 0.589 ms.
+// Complex128 factors, whose products are bound by the FP64 pipe at any size, keep L21:
 //   forward  (leaves -> root):  z = Linv * acc[own];         acc[upd] -= L21 * z   (scatter)
 //   backward (root -> leaves):  v = Dinv z - L21^T x[upd];   x[own]   = Linv^T * v
 // Every block computes a TILE-row slab of one product for a chunk of CC right-hand-side columns
@@ -361,15 +362,14 @@ void launch_level(const Batch& b, int h, int mode, int ldc, cudaStream_t st) {
 }
 
 // One launch for the vectors of all layers (a memset node per layer costs a launch each: 2 x 16
-// of them per substitution at 16 layers; clearing whole vectors took 31 of 943 ms of a 128^3 solve with
-// 32 columns, the rows of split reductions are a tenth of them).  16-byte stores, grid-stride; HBM/L2 write bound.
+// of them per substitution at 16 layers; the rows of split reductions, all that M21 substitutions clear, are a
+// tenth of the vectors).  16-byte stores, grid-stride; HBM/L2 write bound: 15 us a launch at 64^3, 16 columns.
 __global__ void __launch_bounds__(256) k_zero(const ZeroDev* d) {
     const ZeroDev z = d[blockIdx.y];
     float4* p = (float4*)z.p;
     const long long n16 = z.bytes / 16;
     for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n16; i += (long long)gridDim.x * 256)
         p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (blockIdx.x == 0 && threadIdx.x == 0 && (z.bytes & 8)) ((double*)z.p)[2 * n16] = 0.0;
 }
 
 // Records a CUDA event pair around one launch in profiling detail mode.
@@ -726,7 +726,7 @@ BatchLists batch_lists(const Ctx& ctx, const std::vector<int>& layers, size_t el
                         } else {
                             for (int t = 0; t < out_t; ++t) {
                                 if (mode == 0) add_tasks(lists[0][hl], jq, nid, t, 0, t + 1, ks);      // FA: Linv row tile t
-                                if (mode == 1) add_tasks(lists[1][hl], jq, nid, t, 0, nd.own_t, ks);   // FB: L21 row tile t
+                                if (mode == 1) add_tasks(lists[1][hl], jq, nid, t, 0, nd.own_t, ks);   // FB: M21 (L21) row tile t
                                 if (mode == 2) add_tasks(lists[2][hl], jq, nid, t, 0, nd.upd_t, ks);   // BA (>= 1 task)
                                 if (mode == 3) add_tasks(lists[3][hl], jq, nid, t, t, nd.own_t, ks);   // BB
                             }

@@ -15,8 +15,8 @@
 // it is an option (HZ_PRECOND_SPLIT=1) for the local solves inside the preconditioner, whose
 // accuracy changes how fast GMRES converges but not the solution it converges to.
 //
-// Warp-specialized pipeline (16 complex reduction indices per stage, two-deep rings of raw and
-// converted buffers, every hand-off an mbarrier):
+// Warp-specialized pipeline (16 complex reduction indices per stage, rings of two to six raw and two or
+// four converted buffers, every hand-off an mbarrier):
 //   4 loader warps    : cp.async 16-byte copies of the factor tiles and vector rows into a raw
 //                       buffer (masked rows / absent tiles zero-filled by the copy), completion
 //                       signalled with cp.async.mbarrier.arrive;
