@@ -63,3 +63,15 @@ def test_unreachable_tolerance_uses_its_passes(problem):
     from paper_1801_08655_gb300 import hz
     worst, n, status = solve(problem, 1e-30, 4)
     assert n == 4 and status == hz.HZ_ERR_NO_CONVERGENCE and np.isfinite(worst)
+
+
+def test_solution_that_is_not_finite_is_not_converged(problem):
+    """Sources beyond the range of the complex64 local solves: the residual is not a number, which no
+    comparison with refine_tol may pass for converged."""
+    from paper_1801_08655_gb300 import hz
+    s, f = problem
+    with pytest.raises(hz.HzError) as e:
+        s.solve(f * 1e60, hz.default_opts("mixed"))
+    assert e.value.status == hz.HZ_ERR_NONFINITE
+    u = s.solve(f, hz.default_opts("mixed"))[0]           # the handle solves on
+    assert bool(torch.isfinite(u.real).all())
